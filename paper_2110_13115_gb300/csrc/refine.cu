@@ -3,7 +3,20 @@
 // and an in-kernel gradient ascent. The matched filter is Eq. (1) of arXiv:2110.13115 evaluated at
 // t_0 = t_c (Eq. 3-4); the paper stops at the triggers, so the ascent rule is this library's own
 // (see include/rbmf.h). One CTA per candidate recomputes the whitened template frequency by
-// frequency in every pass: Psi in FP64 reduced modulo 2 pi, sin/cos in FP32, sums in FP64.
+// frequency in every pass.
+//
+// Arithmetic. The GPU does two FP64 operations per clock and SM against 128 in FP32, and a point took about 90 of
+// them (four divisions among them). FP64 is left to the phase, which needs it (Psi reaches 1e5 rad and more and is
+// rounded to FP32 only after its reduction modulo 2 pi), in 16 operations: 1 / v comes from a table of 1 / vf and one
+// Newton step that rounds it correctly, 2 pi f from a table, the reduction multiplies by 1 / (2 pi). The rest runs in FP32
+// pairs (an unevaluated sum hi + lo, 48 bits; the products and sums are the classical error-free ones): the term
+// amp s_hat e^(i Psi), and its sums. The derivatives of Psi are linear in f, F5 = (pi f)^(-5/3), F3 = (pi f)^(-1) and
+// F2 = (pi f)^(-2/3) with coefficients that are constant over the points, so a pass sums the terms and their moments
+// with those four, and one thread forms the gradient.
+// Measured (FP64 issue bounds it, 16 operations a point): 512 candidates x 20 steps at n = 2^17 3.35 ms against
+// 17.8 ms with every point in FP64; value and gradient of 500 candidates at n = 2^19 1.61 ms against 5.11 ms. A phase in
+// pairs too would take 1.45 ms and 0.65 ms and is as accurate, but it rounds to another FP32 phase at one
+// point in some thousands, which the ascent amplifies to 1e-8 of J against the FP64 phase.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -18,17 +31,31 @@ constexpr double kMsunS = 4.925491025543576e-06;
 constexpr double kPi = 3.14159265358979323846;
 constexpr double kFref = 100.0;
 constexpr double kEtaMin = 0.05;
-constexpr int kThreads = 256;
+constexpr int kThreads = 128;
 
 enum { R_EVAL = 0, R_ADJOINT = 1, R_ASCEND = 2 };
 
+// Workspace header: flags, the smallest PSD value of the band (complemented bits, so that zero is "none"),
+// the first frequency above every candidate's support.
+struct Header {
+  unsigned flags, jmax;
+  unsigned long long smin;
+};
+
 struct RefArgs {
   const float2* shat;
-  const double* amp;  // f^(-7/6) sqrt(4 df / S_j)
-  const double* vf;   // (pi f_j)^(1/3)
-  int64_t half;
+  const double* psd;
+  Header* head;
+  float4* w;      // amp s_hat as pairs: (re hi, im hi, re lo, im lo), amp = 2^scale f^(-7/6) sqrt(4 df / S)
+  double2* v;     // (vf, 1 / vf), vf = (pi f)^(1/3)
+  double* x;      // 2 pi f
+  float4* g;      // (F5 hi, F5 lo, F3 hi, F3 lo)
+  float2* g2;     // (F2 hi, F2 lo)
+  double* amp2;   // amp^2, zero below the band
+  double* chunk;  // sums of amp2 over blocks of kThreads frequencies
+  int64_t half, jlo;
   double df;
-  double f_low;
+  double p53, p23;  // pi^(-5/3), pi^(-2/3)
   int pn;
   const double* theta_in;
   double* theta_out;
@@ -39,105 +66,306 @@ struct RefArgs {
   int64_t n_cand;
   int steps;
   double alpha0, alpha_max;
-  unsigned* flags;
 };
 
-__global__ void k_refine_tables(int64_t half, double df, const double* psd, double* amp, double* vf, unsigned* flags) {
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < half; j += (int64_t)gridDim.x * blockDim.x) {
-    if (j == 0) {
-      amp[0] = 0.0;
-      vf[0] = 0.0;
+// --- pairs ------------------------------------------------------------------------------------
+struct Pair {
+  float h, l;
+};
+__device__ __forceinline__ Pair to_pair(double x) {
+  const float h = (float)x;
+  return {h, isfinite(h) ? (float)(x - (double)h) : 0.f};
+}
+// s + e = a + b exactly (Knuth)
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+  return s;
+}
+// Sums are kept in three parts: a pair's low part collects the rounding errors of every addition, and its own
+// rounding would cost a digit and a half over a pass (1.6e-14 of the terms' norm against 2e-15).
+struct Sum {
+  float h, m, l;
+};
+__device__ __forceinline__ void add(Sum& s, float h, float l) {
+  float e1, e2, e3;
+  s.h = two_sum(s.h, h, e1);
+  const float x = two_sum(e1, l, e2);
+  s.m = two_sum(s.m, x, e3);
+  s.l = __fadd_rn(s.l, __fadd_rn(e2, e3));
+}
+__device__ __forceinline__ Sum shuffle_xor(const Sum& s, int off) {
+  return {__shfl_xor_sync(0xffffffffu, s.h, off), __shfl_xor_sync(0xffffffffu, s.m, off), __shfl_xor_sync(0xffffffffu, s.l, off)};
+}
+__device__ __forceinline__ void add(Sum& s, const Sum& o) {
+  add(s, o.h, o.m);
+  s.l = __fadd_rn(s.l, o.l);
+}
+__device__ __forceinline__ Pair mul(Pair a, float bh, float bl) {
+  const float p = __fmul_rn(a.h, bh);
+  return {p, __fmaf_rn(a.l, bh, __fmaf_rn(a.h, bl, __fmaf_rn(a.h, bh, -p)))};
+}
+
+// The scale of the amplitudes: a power of two that brings the largest of them (at the lowest frequency and the
+// smallest PSD value, were they together) to about one, whatever the units of the strain.
+__device__ __forceinline__ int amp_scale(const RefArgs& a) {
+  const int ex = (int)((~a.head->smin >> 52) & 2047) - 1023;
+  const float flo = (float)a.jlo * (float)a.df;
+  return -(int)floorf(0.5f * (log2f(4.f * (float)a.df) - (float)ex) - 7.f / 6.f * log2f(flo)) - 1;
+}
+
+// PSD check (0 < j < half), the band's smallest value, and the end of the candidates' supports (an FP32
+// estimate with a margin: it only bounds the tables).
+__global__ void __launch_bounds__(kThreads) k_refine_check(RefArgs a) {
+  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+  unsigned long long low = 0;
+  bool bad = false;
+  for (int64_t j = tid + 1; j < a.half; j += stride) {
+    const double S = a.psd[j];
+    if (!(S > 0.0) || isinf(S)) bad = true;
+    else if (j >= a.jlo) low = max(low, ~(unsigned long long)__double_as_longlong(S));
+  }
+  unsigned top = 0;
+  for (int64_t c = tid; c < a.n_cand; c += stride) {
+    const float mc = (float)a.theta_in[4 * c], eta = (float)a.theta_in[4 * c + 1];
+    if (!(mc > 0.f) || !(eta > 0.f)) {  // (or below FP32: the whole band; an invalid candidate is refused later)
+      top = (unsigned)a.half;
       continue;
     }
-    const double f = j * df, S = psd[j];
-    if (!(S > 0.0) || isinf(S) || isnan(S)) {
-      atomicOr(flags, (unsigned)RB_FLAG_BAD_PSD);
-      amp[j] = 0.0;
-    } else {
-      amp[j] = pow(f, -7.0 / 6.0) * sqrt(4.0 * df / S);
+    const float fcut = 1.001f / (14.6969385f * (float)kPi * mc * powf(eta, -0.6f) * (float)kMsunS);
+    top = max(top, (unsigned)fminf((float)a.half, fcut / (float)a.df + 4.f));
+  }
+  for (int off = 16; off > 0; off >>= 1) {
+    low = max(low, __shfl_xor_sync(0xffffffffu, low, off));
+    top = max(top, __shfl_xor_sync(0xffffffffu, top, off));
+  }
+  bad = __any_sync(0xffffffffu, bad);
+  if ((threadIdx.x & 31) == 0) {
+    if (low) atomicMax(&a.head->smin, low);
+    if (top) atomicMax(&a.head->jmax, top);
+    if (bad) atomicOr(&a.head->flags, (unsigned)RB_FLAG_BAD_PSD);
+  }
+}
+
+// Sum over the block of one double per thread (every thread calls; the result on thread 0 only).
+__device__ __forceinline__ double block_sum(double v, double* red) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int w = 1; w < kThreads / 32; ++w) v += red[w];
+  return v;
+}
+
+// The tables on [jlo, jmax): everything is a power of y = f^(-1/6) (an FP32 estimate and two Newton steps in
+// FP64: the error 3.5 e^2 of a step takes 1e-6 below the rounding of FP64).
+__global__ void __launch_bounds__(kThreads) k_refine_tables(RefArgs a) {
+  __shared__ double red[kThreads / 32];
+  const int64_t jmax = min((int64_t)a.head->jmax, a.half);
+  const double scale = scalbn(2.0 * sqrt(a.df), amp_scale(a));
+  for (int64_t c = a.jlo / kThreads + blockIdx.x; c * kThreads < jmax; c += gridDim.x) {
+    const int64_t j = c * kThreads + threadIdx.x;
+    double a2 = 0.0;
+    if (j >= a.jlo && j < jmax) {
+      const double f = j * a.df;
+      double y = (double)exp2f(log2f((float)f) * (-1.f / 6.f));
+#pragma unroll
+      for (int it = 0; it < 2; ++it) {
+        const double y2 = y * y, y6 = y2 * y2 * y2;
+        y = y * (fma(-f, y6, 7.0) * (1.0 / 6.0));
+      }
+      const double y2 = y * y, y4 = y2 * y2, y6 = y4 * y2, y10 = y6 * y4;
+      const double am = scale * (y6 * y) * rsqrt(a.psd[j]);
+      const float2 sh = a.shat[j];
+      const Pair re = to_pair(am * (double)sh.x), im = to_pair(am * (double)sh.y);
+      const Pair f5 = to_pair(a.p53 * y10), f3 = to_pair(y6 * (1.0 / kPi)), f2 = to_pair(a.p23 * y4);
+      const double vf = cbrt(kPi * f);
+      a.v[j] = make_double2(vf, 1.0 / vf);
+      a.x[j] = 2.0 * kPi * f;
+      a.w[j] = make_float4(re.h, im.h, re.l, im.l);
+      a.g[j] = make_float4(f5.h, f5.l, f3.h, f3.l);
+      a.g2[j] = make_float2(f2.h, f2.l);
+      a2 = am * am;
     }
-    vf[j] = cbrt(kPi * f);
+    if (j < a.half) a.amp2[j] = a2;
+    a2 = block_sum(a2, red);
+    if (threadIdx.x == 0) a.chunk[c] = a2;
   }
 }
 
-// Sum NV doubles over the block; every thread receives the totals.
-template <int NV>
-__device__ __forceinline__ void block_sum(double (&v)[NV], double* red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int i = 0; i < NV; ++i)
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], off);
-  __syncthreads();
-  if (lane == 0)
-#pragma unroll
-    for (int i = 0; i < NV; ++i) red[warp * NV + i] = v[i];
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < NV; ++i) {
-    double s = 0.0;
-    for (int w = 0; w < kThreads / 32; ++w) s += red[w * NV + i];
-    v[i] = s;
-  }
-}
+// --- one pass over the frequencies ---------------------------------------------------------------
+// A candidate's constants (from one thread, by way of shared memory).
+struct Point {
+  double m13, r13, c0, c2, c3, tc, phic;  // v = m13 vf, r13 = 1 / m13; Psi's coefficients
+  // coefficients of the moments in dPsi/dmc (F5, F3, F2) and dPsi/deta (F3, F2)
+  double m5, m3, m2, e3, e2;
+};
 
-// Z (v[0..1]) and, when GRAD, dZ/dtheta_k (v[2 + 2k .. 3 + 2k]) summed over [jlo, jhi).
-template <bool GRAD>
-__device__ void evaluate(const RefArgs& a, const double (&th)[4], int64_t jlo, int64_t jhi, double (&v)[10],
-                         double* red) {
+__device__ void make_point(const RefArgs& a, const double (&th)[4], Point& p) {
   const double mc = th[0], eta = th[1], tc = th[2], phic = th[3];
-  const double mt = mc * pow(eta, -0.6) * kMsunS;
-  const double m13 = cbrt(mt);
-  const double c0 = 3.0 / (128.0 * eta);
   const double c2 = a.pn >= 2 ? (20.0 / 9.0) * (743.0 / 336.0 + 11.0 * eta / 4.0) : 0.0;
-  const double c3 = a.pn >= 3 ? -16.0 * kPi : 0.0;
   const double dc2 = a.pn >= 2 ? (20.0 / 9.0) * (11.0 / 4.0) : 0.0;
+  const double c3 = a.pn >= 3 ? -16.0 * kPi : 0.0;
+  const double mt = mc * pow(eta, -0.6) * kMsunS;
+  p.m13 = cbrt(mt);
+  p.r13 = 1.0 / p.m13;
+  p.c0 = 3.0 / (128.0 * eta);
+  p.c2 = c2;
+  p.c3 = c3;
+  p.tc = tc;
+  p.phic = phic;
+  // Psi = A5 F5 + A3 F3 + A2 F2
+  const double r2 = p.r13 * p.r13, a5 = p.c0 * (r2 * r2 * p.r13), a3 = p.c0 * c2 * (r2 * p.r13), a2 = p.c0 * c3 * r2;
+  p.m5 = -5.0 / 3.0 * a5 / mc;
+  p.m3 = -a3 / mc;
+  p.m2 = -2.0 / 3.0 * a2 / mc;
+  p.e3 = p.c0 * (r2 * p.r13) * (dc2 - 0.4 * c2 / eta);
+  p.e2 = -0.6 * a2 / eta;
+}
+
+// The sums of a pass (thread 0 after evaluate): Z and the moments with j, F5, F3, F2.
+struct Sums {
+  double z[2], s1[2], m5[2], m3[2], m2[2];
+};
+
+// Sums of V values over a warp into out[V]: halves of the list are exchanged while there is more than one value left.
+template <int V>
+__device__ __forceinline__ void warp_sums(Sum (&v)[V], double* out) {
+  const int lane = threadIdx.x & 31;
+  int first = 0;
 #pragma unroll
-  for (int i = 0; i < 10; ++i) v[i] = 0.0;
-  for (int64_t j = jlo + threadIdx.x; j < jhi; j += blockDim.x) {
-    const double f = j * a.df;
-    const double vv = m13 * a.vf[j];
-    const double iv = 1.0 / vv, iv2 = iv * iv, iv3 = iv2 * iv, iv5 = iv3 * iv2;
-    const double psi_pn = c0 * (iv5 + c2 * iv3 + c3 * iv2);
-    double psi = 2.0 * kPi * f * tc - phic - 0.25 * kPi + psi_pn;
-    psi -= 2.0 * kPi * rint(psi / (2.0 * kPi));
+  for (int step = 0, keep = V / 2; step < 5; ++step, keep /= 2) {
+    const int off = 16 >> step;
+    const bool up = (lane & off) != 0;
+    if (keep > 0) {
+      first += up ? keep : 0;
+#pragma unroll
+      for (int i = 0; i < keep; ++i) {
+        const Sum give = up ? v[i] : v[i + keep];
+        v[i] = up ? v[i + keep] : v[i];
+        add(v[i], shuffle_xor(give, off));
+      }
+    } else {
+      add(v[0], shuffle_xor(v[0], off));
+    }
+  }
+  constexpr int kCopies = 32 / V;  // lanes that hold the same value
+  if ((lane & (kCopies - 1)) == 0) out[first] = (double)v[0].h + ((double)v[0].m + (double)v[0].l);
+}
+
+template <bool GRAD, bool PN3>
+__device__ void evaluate(const RefArgs& a, const Point* shared, int64_t jhi, double* red, Sums& out) {
+  constexpr int V = GRAD ? 8 : 2;
+  const double m13 = shared->m13, r13 = shared->r13, c0 = shared->c0, c2 = shared->c2, c3 = shared->c3, tc = shared->tc,
+               phic = shared->phic;
+  Sum v[V] = {}, v2[2] = {};
+#pragma unroll 2
+  for (int64_t j = a.jlo + threadIdx.x; j < jhi; j += kThreads) {
+    const float4 w = __ldg(a.w + j);
+    const double2 vt = __ldg(a.v + j);
+    const double vv = m13 * vt.x, guess = r13 * vt.y;  // 1 / vv within two units in the last place
+    const double iv = fma(guess, fma(-vv, guess, 1.0), guess);
+    const double iv2 = iv * iv, iv3 = iv2 * iv, iv5 = iv3 * iv2;
+    const double psi_pn = PN3 ? c0 * (iv5 + c2 * iv3 + c3 * iv2) : c0 * (iv5 + c2 * iv3);
+    double phase = __ldg(a.x + j) * tc - phic - 0.25 * kPi + psi_pn;
+    // the nearest whole number of turns, by an addition that leaves no fraction bits (|turns| < 2^51)
+    const double k = fma(phase, 1.0 / (2.0 * kPi), 6755399441055744.0) - 6755399441055744.0;
+    phase -= 2.0 * kPi * k;
+    const float psi = (float)phase;
     float sn, cs;
-    sincosf((float)psi, &sn, &cs);
-    const float2 sh = a.shat[j];
-    const double am = a.amp[j];
-    // term = s_hat * conj(g) = s_hat * amp * exp(+i Psi)
-    const double tr = am * ((double)sh.x * cs - (double)sh.y * sn);
-    const double ti = am * ((double)sh.x * sn + (double)sh.y * cs);
-    v[0] += tr;
-    v[1] += ti;
-    if (GRAD) {
-      const double dpsi_dm = (-5.0 * iv5 - 3.0 * c2 * iv3 - 2.0 * c3 * iv2) / (128.0 * eta * mt);
-      const double dpsi_deta_m = -psi_pn / eta + c0 * dc2 * iv3;
-      const double d[4] = {dpsi_dm * mt / mc, dpsi_deta_m + dpsi_dm * (-0.6 * mt / eta), 2.0 * kPi * f, -1.0};
+    sincosf(psi, &sn, &cs);
+    // term = w exp(i Psi)
+    Pair t[2];
+    float e;
+    {
+      const float p = __fmul_rn(w.x, cs), q = __fmul_rn(w.y, sn);
+      t[0].h = two_sum(p, -q, e);
+      t[0].l = __fadd_rn(e, __fsub_rn(__fmaf_rn(w.z, cs, __fmaf_rn(w.x, cs, -p)), __fmaf_rn(w.w, sn, __fmaf_rn(w.y, sn, -q))));
+    }
+    {
+      const float p = __fmul_rn(w.x, sn), q = __fmul_rn(w.y, cs);
+      t[1].h = two_sum(p, q, e);
+      t[1].l = __fadd_rn(e, __fadd_rn(__fmaf_rn(w.z, sn, __fmaf_rn(w.x, sn, -p)), __fmaf_rn(w.w, cs, __fmaf_rn(w.y, cs, -q))));
+    }
+    float4 g;
+    float2 g2;
+    if constexpr (GRAD) g = __ldg(a.g + j);
+    if constexpr (GRAD && PN3) g2 = __ldg(a.g2 + j);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {  // i d term
-        v[2 + 2 * k] -= d[k] * ti;
-        v[3 + 2 * k] += d[k] * tr;
+    for (int c = 0; c < 2; ++c) {
+      add(v[c], t[c].h, t[c].l);
+      if constexpr (GRAD) {
+        const float fj = (float)(int)j;  // exact
+        const float p = __fmul_rn(t[c].h, fj);
+        add(v[2 + c], p, __fmaf_rn(t[c].l, fj, __fmaf_rn(t[c].h, fj, -p)));
+        const Pair x5 = mul(t[c], g.x, g.y), x3 = mul(t[c], g.z, g.w);
+        add(v[4 + c], x5.h, x5.l);
+        add(v[6 + c], x3.h, x3.l);
+        if constexpr (PN3) {
+          const Pair x2 = mul(t[c], g2.x, g2.y);
+          add(v2[c], x2.h, x2.l);
+        }
       }
     }
   }
-  block_sum<10>(v, red);
+  // block sums: pairs within a warp, FP64 across the warps
+  constexpr int NV = GRAD && PN3 ? V + 2 : V;
+  __syncthreads();  // (red may still be read from the pass before)
+  warp_sums<V>(v, red + (threadIdx.x >> 5) * NV);
+  if constexpr (GRAD && PN3) warp_sums<2>(v2, red + (threadIdx.x >> 5) * NV + V);
+  __syncthreads();
+  if (threadIdx.x < NV) {
+    double t = red[threadIdx.x];
+    for (int k = 1; k < kThreads / 32; ++k) t += red[k * NV + threadIdx.x];
+    red[threadIdx.x] = t;  // (only this thread reads this column)
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    out.z[0] = red[0];
+    out.z[1] = red[1];
+    if constexpr (GRAD) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        out.s1[c] = red[2 + c];
+        out.m5[c] = red[4 + c];
+        out.m3[c] = red[6 + c];
+        out.m2[c] = PN3 ? red[8 + c] : 0.0;
+      }
+    }
+  }
 }
 
-__device__ __forceinline__ void support(const RefArgs& a, double mc0, double eta0, int64_t& jlo, int64_t& jhi) {
+// Re(conj(zeta) dZ/dtheta_k) for zeta = (zr, zi), dZ/dtheta_k = i sum dPsi_k term (thread 0)
+__device__ __forceinline__ void derivatives(const RefArgs& a, const Point& p, const Sums& s, double zr, double zi, double (&d)[4]) {
+  double t[3][2];
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    t[0][c] = p.m5 * s.m5[c] + p.m3 * s.m3[c] + p.m2 * s.m2[c];
+    t[1][c] = p.e3 * s.m3[c] + p.e2 * s.m2[c];
+    t[2][c] = 2.0 * kPi * a.df * s.s1[c];
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) d[k] = zi * t[k][0] - zr * t[k][1];
+  d[3] = zr * s.z[1] - zi * s.z[0];  // dPsi/dphi_c = -1
+}
+
+__device__ __forceinline__ int64_t support_end(const RefArgs& a, double mc0, double eta0) {
   const double mt0 = mc0 * pow(eta0, -0.6) * kMsunS;
   const double fcut = 1.0 / (pow(6.0, 1.5) * kPi * mt0);
-  jlo = (int64_t)floor(a.f_low / a.df) - 1;
-  if (jlo < 1) jlo = 1;
-  while (jlo < a.half && (double)jlo * a.df < a.f_low) ++jlo;
-  jhi = (int64_t)floor(fcut / a.df) + 2;
-  if (jhi > a.half) jhi = a.half;
-  while (jhi > jlo && (double)(jhi - 1) * a.df >= fcut) --jhi;
+  const double top = floor(fcut / a.df) + 2.0;  // (before the cast: a tiny mass puts it beyond 64 bits)
+  int64_t jhi = top < (double)a.half ? (int64_t)top : a.half;
+  while (jhi > a.jlo && (double)(jhi - 1) * a.df >= fcut) --jhi;
+  return max(jhi, a.jlo);
 }
 
-template <int MODE>
-__global__ void __launch_bounds__(kThreads) k_refine(RefArgs a) {
+template <int MODE, bool PN3>
+__global__ void __launch_bounds__(kThreads, 4) k_refine(RefArgs a) {
   __shared__ double red[(kThreads / 32) * 10];
+  __shared__ Point point;
+  __shared__ int64_t s_jhi;
+  __shared__ int s_go;
   const int64_t c = blockIdx.x;
   if (c >= a.n_cand) return;
   double th[4];
@@ -145,68 +373,84 @@ __global__ void __launch_bounds__(kThreads) k_refine(RefArgs a) {
   for (int i = 0; i < 4; ++i) th[i] = a.theta_in[4 * c + i];
   if (!(th[0] > 0.0) || !(th[1] > 0.0) || !(th[1] <= 0.25) || !isfinite(th[2]) || !isfinite(th[3])) {
     if (threadIdx.x == 0) {
-      atomicOr(a.flags, (unsigned)RB_FLAG_BAD_STRAIN);
+      atomicOr(&a.head->flags, (unsigned)RB_FLAG_BAD_STRAIN);
       if (a.J) a.J[c] = __longlong_as_double(0x7ff8000000000000ll);
     }
     return;
   }
-  int64_t jlo, jhi;
-  support(a, th[0], th[1], jlo, jhi);
-  double s2[1] = {0.0};
-  for (int64_t j = jlo + threadIdx.x; j < jhi; j += blockDim.x) s2[0] += a.amp[j] * a.amp[j];
-  block_sum<1>(s2, red);
-  const double sig2 = s2[0];
-  double v[10];
+  if (threadIdx.x == 0) s_jhi = support_end(a, th[0], th[1]);
+  if (threadIdx.x == 32) make_point(a, th, point);
+  __syncthreads();
+  const int64_t jhi = min(s_jhi, (int64_t)a.head->jmax);
+  // sigma^2 from the chunk sums and the last chunk's part
+  double s2 = 0.0;
+  const int64_t whole = jhi / kThreads;
+  for (int64_t k = a.jlo / kThreads + threadIdx.x; k < whole; k += kThreads) s2 += a.chunk[k];
+  if (whole * kThreads + threadIdx.x < jhi && whole * kThreads + threadIdx.x >= a.jlo) s2 += a.amp2[whole * kThreads + threadIdx.x];
+  const double sig2 = block_sum(s2, red);  // (thread 0)
+  Sums s;
   if (MODE == R_EVAL) {
-    evaluate<false>(a, th, jlo, jhi, v, red);
+    evaluate<false, PN3>(a, &point, jhi, red, s);
     if (threadIdx.x == 0) {
-      a.J[c] = (v[0] * v[0] + v[1] * v[1]) / sig2;
-      a.Z[2 * c] = v[0];
-      a.Z[2 * c + 1] = v[1];
+      const double unit = scalbn(1.0, -amp_scale(a));
+      a.J[c] = (s.z[0] * s.z[0] + s.z[1] * s.z[1]) / sig2;
+      a.Z[2 * c] = s.z[0] * unit;
+      a.Z[2 * c + 1] = s.z[1] * unit;
     }
   } else if (MODE == R_ADJOINT) {
-    evaluate<true>(a, th, jlo, jhi, v, red);
-    const double zr = a.Z[2 * c], zi = a.Z[2 * c + 1], g = a.dJ[c];
-    if (threadIdx.x == 0)
+    evaluate<true, PN3>(a, &point, jhi, red, s);
+    if (threadIdx.x == 0) {
+      const double unit = scalbn(1.0, amp_scale(a)), g = a.dJ[c];
+      double d[4];
+      derivatives(a, point, s, a.Z[2 * c] * unit, a.Z[2 * c + 1] * unit, d);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) a.dtheta[4 * c + k] = g * 2.0 * (zr * v[2 + 2 * k] + zi * v[3 + 2 * k]) / sig2;
+      for (int k = 0; k < 4; ++k) a.dtheta[4 * c + k] = g * 2.0 * d[k] / sig2;
+    }
   } else {
     const double scale[4] = {th[0], 1.0, 1.0 / kFref, 1.0};
-    double u[4], grad[4];
+    double u[4], ut[4], grad[4], J = 0.0, alpha = a.alpha0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) u[k] = th[k] / scale[k];
-    evaluate<true>(a, th, jlo, jhi, v, red);
-    double J = (v[0] * v[0] + v[1] * v[1]) / sig2;
+    for (int step = -1; step < a.steps; ++step) {  // step -1: the starting point
+      if (step >= 0) {
+        if (threadIdx.x == 0) {
+          double gu[4], nrm = 0.0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) grad[k] = 2.0 * (v[0] * v[2 + 2 * k] + v[1] * v[3 + 2 * k]) / sig2;
-    double alpha = a.alpha0;
-    for (int step = 0; step < a.steps; ++step) {
-      double gu[4], nrm = 0.0;
+          for (int k = 0; k < 4; ++k) {
+            gu[k] = grad[k] * scale[k];
+            nrm += gu[k] * gu[k];
+          }
+          nrm = sqrt(nrm);
+          s_go = nrm > 0.0;
+          if (nrm > 0.0) {
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        gu[k] = grad[k] * scale[k];
-        nrm += gu[k] * gu[k];
-      }
-      nrm = sqrt(nrm);
-      if (!(nrm > 0.0)) continue;
-      double ut[4], tt[4];
+            for (int k = 0; k < 4; ++k) ut[k] = u[k] + alpha * gu[k] / nrm;
+            ut[1] = fmin(fmax(ut[1], kEtaMin), 0.25);
+            double tt[4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) ut[k] = u[k] + alpha * gu[k] / nrm;
-      ut[1] = fmin(fmax(ut[1], kEtaMin), 0.25);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) tt[k] = ut[k] * scale[k];
-      evaluate<true>(a, tt, jlo, jhi, v, red);
-      const double Jt = (v[0] * v[0] + v[1] * v[1]) / sig2;
-      if (Jt > J) {
-        J = Jt;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          u[k] = ut[k];
-          grad[k] = 2.0 * (v[0] * v[2 + 2 * k] + v[1] * v[3 + 2 * k]) / sig2;
+            for (int k = 0; k < 4; ++k) tt[k] = ut[k] * scale[k];
+            make_point(a, tt, point);
+          }
         }
-        alpha = fmin(2.0 * alpha, a.alpha_max);
-      } else {
-        alpha *= 0.5;
+        __syncthreads();
+        if (!s_go) break;  // (the gradient stays what it is)
+      }
+      evaluate<true, PN3>(a, &point, jhi, red, s);
+      if (threadIdx.x == 0) {
+        const double Jt = (s.z[0] * s.z[0] + s.z[1] * s.z[1]) / sig2;
+        if (step < 0 || Jt > J) {
+          J = Jt;
+          double d[4];
+          derivatives(a, point, s, s.z[0], s.z[1], d);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            if (step >= 0) u[k] = ut[k];
+            grad[k] = 2.0 * d[k] / sig2;
+          }
+          if (step >= 0) alpha = fmin(2.0 * alpha, a.alpha_max);
+        } else {
+          alpha *= 0.5;
+        }
       }
     }
     if (threadIdx.x == 0) {
@@ -218,6 +462,25 @@ __global__ void __launch_bounds__(kThreads) k_refine(RefArgs a) {
 }
 
 size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
+
+// Workspace: header, then the tables over the frequencies. base == nullptr: only the size.
+size_t carve(int64_t half, char* base, RefArgs* a) {
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    char* p = base ? base + off : nullptr;
+    off += a256(bytes);
+    return p;
+  };
+  a->head = (Header*)take(256);
+  a->w = (float4*)take(sizeof(float4) * half);
+  a->v = (double2*)take(sizeof(double2) * half);
+  a->x = (double*)take(sizeof(double) * half);
+  a->g = (float4*)take(sizeof(float4) * half);
+  a->g2 = (float2*)take(sizeof(float2) * half);
+  a->amp2 = (double*)take(sizeof(double) * half);
+  a->chunk = (double*)take(sizeof(double) * ((half + kThreads - 1) / kThreads));
+  return off;
+}
 
 int prepare(const rb_refine_desc* d, const float* shat, const double* psd, const void* theta, int64_t n_cand,
             void* ws, size_t bytes, RefArgs& a, cudaStream_t st) {
@@ -237,22 +500,27 @@ int prepare(const rb_refine_desc* d, const float* shat, const double* psd, const
     return RB_ERR_OOM;
   }
   const int64_t half = d->n / 2;
-  char* base = (char*)ws;
-  a.flags = (unsigned*)base;
-  a.amp = (const double*)(base + 256);
-  a.vf = (const double*)(base + 256 + a256(sizeof(double) * half));
+  carve(half, (char*)ws, &a);
   a.shat = (const float2*)shat;
+  a.psd = psd;
+  a.theta_in = (const double*)theta;
   a.half = half;
   a.df = d->fs / (double)d->n;
-  a.f_low = d->f_low;
+  // first frequency of the band: j >= 1, j df >= f_low
+  const double low = std::floor(d->f_low / a.df) - 1.0;
+  a.jlo = low < 1.0 ? 1 : low < (double)half ? (int64_t)low : half;
+  while (a.jlo < half && (double)a.jlo * a.df < d->f_low) ++a.jlo;
+  a.p53 = std::pow(kPi, -5.0 / 3.0);
+  a.p23 = std::pow(kPi, -2.0 / 3.0);
   a.pn = d->pn_order;
   a.n_cand = n_cand;
   a.steps = d->steps;
   a.alpha0 = d->alpha0;
   a.alpha_max = d->alpha_max;
-  RB_CUDA_TRY(cudaMemsetAsync(a.flags, 0, 256, st));
-  k_refine_tables<<<(int)std::min<int64_t>(1024, (half + 255) / 256), 256, 0, st>>>(
-      half, a.df, psd, (double*)a.amp, (double*)a.vf, a.flags);
+  RB_CUDA_TRY(cudaMemsetAsync(a.head, 0, 256, st));
+  k_refine_check<<<(int)std::min<int64_t>(304, (half + kThreads - 1) / kThreads), kThreads, 0, st>>>(a);
+  RB_LAUNCH_CHECK();
+  k_refine_tables<<<(int)std::min<int64_t>(1216, (half + kThreads - 1) / kThreads), kThreads, 0, st>>>(a);
   RB_LAUNCH_CHECK();
   return RB_OK;
 }
@@ -260,11 +528,14 @@ int prepare(const rb_refine_desc* d, const float* shat, const double* psd, const
 template <int MODE>
 int run(const RefArgs& a, cudaStream_t st) {
   if (a.n_cand > 0) {
-    k_refine<MODE><<<(unsigned)a.n_cand, kThreads, 0, st>>>(a);
+    if (a.pn >= 3)
+      k_refine<MODE, true><<<(unsigned)a.n_cand, kThreads, 0, st>>>(a);
+    else
+      k_refine<MODE, false><<<(unsigned)a.n_cand, kThreads, 0, st>>>(a);
     RB_LAUNCH_CHECK();
   }
   unsigned flags = 0;
-  RB_CUDA_TRY(cudaMemcpyAsync(&flags, a.flags, sizeof(flags), cudaMemcpyDeviceToHost, st));
+  RB_CUDA_TRY(cudaMemcpyAsync(&flags, &a.head->flags, sizeof(flags), cudaMemcpyDeviceToHost, st));
   RB_CUDA_TRY(cudaStreamSynchronize(st));
   if (flags & RB_FLAG_BAD_PSD) {
     rb::set_detail("PSD not finite and positive on 0 < j < n/2");
@@ -283,7 +554,8 @@ extern "C" {
 
 size_t rb_refine_workspace_bytes(const rb_refine_desc* d) {
   if (!d || d->n < 2) return 0;
-  return 256 + 2 * a256(sizeof(double) * (size_t)(d->n / 2));
+  RefArgs a{};
+  return carve(d->n / 2, nullptr, &a);
 }
 
 int rb_refine_eval(const rb_refine_desc* d, const float* s_hat, const double* psd, const double* theta, double* J,
@@ -296,7 +568,6 @@ int rb_refine_eval(const rb_refine_desc* d, const float* s_hat, const double* ps
     rb::set_detail("NULL output");
     return RB_ERR_BAD_INPUT;
   }
-  a.theta_in = theta;
   a.J = J;
   a.Z = Z;
   return run<R_EVAL>(a, st);
@@ -313,7 +584,6 @@ int rb_refine_adjoint(const rb_refine_desc* d, const float* s_hat, const double*
     rb::set_detail("NULL argument");
     return RB_ERR_BAD_INPUT;
   }
-  a.theta_in = theta;
   a.Z = (double*)Z;
   a.dJ = dJ;
   a.dtheta = dtheta;
@@ -330,7 +600,6 @@ int rb_refine(const rb_refine_desc* d, const float* s_hat, const double* psd, do
     rb::set_detail("NULL output");
     return RB_ERR_BAD_INPUT;
   }
-  a.theta_in = theta;
   a.theta_out = theta;
   a.J = J;
   return run<R_ASCEND>(a, st);
