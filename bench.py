@@ -1140,10 +1140,10 @@ def main():
     else:
         byts = ksum * (half * 8 + half * 8 + nb * 8)
         achieved = byts / (stage_ms[dom] / 1e3) / 1e9
-        roof = dict(bound="hbm", achieved=achieved, peak=hbm, unit="GB/s", kernel="k_pass_a+k_pass_b (basis)",
+        roof = dict(bound="hbm", achieved=achieved, peak=hbm, unit="GB/s", kernel="k_series (basis)",
                     peak_source="MEASURED_PEAKS hbm_gbs", algorithmic_bytes=byts)
-        key, srcs = "basis_filter", ("paper_2110_13115_gb300/csrc/filter.cu", "paper_2110_13115_gb300/csrc/fft.cuh",
-                                     "paper_2110_13115_gb300/csrc/fft2.cuh")
+        key, srcs = "basis_filter", ("paper_2110_13115_gb300/csrc/filter.cu", "paper_2110_13115_gb300/csrc/series.cuh",
+                                     "paper_2110_13115_gb300/csrc/pair.cuh")
     roof["frac"] = roof["achieved"] / roof["peak"]
     roof["traffic"] = traffic_from_profiles(key, source_hash(*srcs), units=ksum if key == "basis_filter" else None)
     roof["stage"] = dom

@@ -161,6 +161,8 @@ int rb_whiten(const rb_filter_desc* desc, const float* strain, const double* psd
  *   beta_avg: [k][n/(2w)] complex output (index i - n/(2w)).
  *   Errors: RB_ERR_BAD_INPUT (desc invalid, basis not matching desc, NULL s_hat or beta_avg),
  *   RB_ERR_OOM (workspace smaller than rb_filter_plan's size or not 256-byte aligned).
+ *   Enqueue only: a bounded device-side wait that gave up (RB_ERR_TIMEOUT of the calls that read the
+ *   status) leaves beta incomplete without a report here.
  */
 int rb_basis_filter(const rb_filter_desc* desc, const rb_basis* basis, const float* s_hat,
                     float* beta, float* beta_avg, void* workspace, size_t workspace_bytes,
@@ -420,8 +422,8 @@ int rb_tune_stage1(const rb_filter_desc* desc, const rb_basis* basis, const floa
 /*
  * rb_tune_fft - autotuner of the FFT schedule of the basis filter (rb_basis_filter, and inside
  * rb_filter / rb_filter_batch / rb_filter_plain): times every variant of RB_FFT_VARIANTS (columns
- * per CTA of the two four-step passes, and the size of the chunk of vectors whose intermediate stays
- * in L2) on this desc's basis and s_hat, and remembers the fastest for (n, w) in a process-wide
+ * per CTA of the two four-step passes of short transforms, and the megabytes of the intermediate that
+ * are to stay in L2) on this desc's basis and s_hat, and remembers the fastest for (n, w) in a process-wide
  * table (variant 0 when untuned). Measurement support, not in the paper.
  *   s_hat: [n/2] complex device (rb_whiten output). times_ms: HOST [RB_FFT_VARIANTS] mean ms of one
  *   basis filter. chosen: HOST, the selected variant. Synchronises `stream`.

@@ -150,19 +150,19 @@ void carve(const rb_filter_desc& d, const Geometry& g, char* base, Workspace* ws
   ws->tables.n2_w = (float2*)take(sizeof(float2) * g.n2);
   ws->tables.fine_w = (float2*)take(sizeof(float2) * g.n2);
   ws->tables.w2a_w = (float2*)take(sizeof(float2) * w2_entries(g.n2));
-  ws->tables.w2b_w = (float2*)take(sizeof(float2) * w2_entries(g.n1));
+  ws->tables.w4_w = (float2*)take(sizeof(float2) * (g.n1 / 4 + 128));
   ws->tables.n1 = ws->tables.n1_w;
   ws->tables.n2 = ws->tables.n2_w;
   ws->tables.fine = ws->tables.fine_w;
   ws->tables.w2a = ws->tables.w2a_w;
-  ws->tables.w2b = ws->tables.w2b_w;
+  ws->tables.w4 = ws->tables.w4_w;
   ws->wt = (float*)take(sizeof(float) * half);
   ws->shat = (float2*)take(sizeof(float2) * half);
+  ws->sync = (unsigned*)take(sizeof(unsigned) * sync_words(g.n));
   // everything above depends on n only, so sub-banks that share a workspace share it
   if (!plain && (d.mem & RB_MEM_HOST_TRIGGERS)) ws->trig_stage = (rb_trigger*)take(host_trig_bytes(g));
   const int64_t nvec = plain ? d.n_templates : d.k;
-  int64_t vc = (int64_t(96) << 20) / (g.n * 8);  // four-step chunks of up to 96 MB (kept in L2)
-  vc = std::max<int64_t>(1, std::min<int64_t>(vc, std::min<int64_t>(nvec, 65535)));
+  const int64_t vc = std::min<int64_t>(max_x_rows(g.n), std::min<int64_t>(nvec, 65535));
   ws->vc = (int)vc;
   ws->X = (float2*)take(sizeof(float2) * g.n * vc);
   if (!plain) {
@@ -266,6 +266,8 @@ struct FoldWs {
   Geometry gn, gm;
   Workspace wn, wm;
   float2* gfold = nullptr;
+  float2* folded = nullptr;  // folded spectra of `rows` templates for the fused transforms
+  int rows = 0;
   size_t total = 0;
 };
 
@@ -307,12 +309,13 @@ void carve_fold(const rb_filter_desc& d, char* base, FoldWs* f) {
     w->tables.n2_w = (float2*)take(sizeof(float2) * g.n2);
     w->tables.fine_w = (float2*)take(sizeof(float2) * g.n2);
     w->tables.w2a_w = (float2*)take(sizeof(float2) * w2_entries(g.n2));
-    w->tables.w2b_w = (float2*)take(sizeof(float2) * w2_entries(g.n1));
+    w->tables.w4_w = (float2*)take(sizeof(float2) * (g.n1 / 4 + 128));
     w->tables.n1 = w->tables.n1_w;
     w->tables.n2 = w->tables.n2_w;
     w->tables.fine = w->tables.fine_w;
     w->tables.w2a = w->tables.w2a_w;
-    w->tables.w2b = w->tables.w2b_w;
+    w->tables.w4 = w->tables.w4_w;
+    w->sync = (unsigned*)take(sizeof(unsigned) * sync_words(g.n));
   };
   tables(&f->wn, gn);
   tables(&f->wm, gm);
@@ -320,11 +323,13 @@ void carve_fold(const rb_filter_desc& d, char* base, FoldWs* f) {
   f->wn.shat = (float2*)take(sizeof(float2) * gn.n / 2);
   f->wm.shat = f->wn.shat;
   f->gfold = (float2*)take(sizeof(float2) * gn.n / 2);
-  int64_t vc = (int64_t(96) << 20) / (gm.n * 8);
-  vc = std::max<int64_t>(1, std::min<int64_t>(vc, std::min<int64_t>(d.n_templates, 65535)));
+  const int64_t vc = std::min<int64_t>(max_x_rows(gm.n), std::min<int64_t>(d.n_templates, 65535));
   f->wm.vc = (int)vc;
   f->wn.vc = 1;
   f->wm.X = f->wn.X = (float2*)take(sizeof(float2) * std::max<int64_t>(gm.n * vc, gn.n));
+  // up to 64 MB of folded spectra, which L2 holds until the transforms have read them
+  f->rows = gm.n >= (1 << 14) ? (int)std::max<int64_t>(1, std::min<int64_t>(d.n_templates, (int64_t(8) << 20) / gm.n)) : 0;
+  f->folded = (float2*)take(sizeof(float2) * gm.n * (size_t)f->rows);
   f->total = off;
 }
 
@@ -459,7 +464,7 @@ int batch_status(const BatchSpec& s, int64_t* n_trig, cudaStream_t st) {
     return RB_ERR_BAD_INPUT;
   }
   if (stt.flags & RB_FLAG_TIMEOUT) {
-    set_detail("a bounded device-side wait (tcgen05 first or second stage) timed out");
+    set_detail("a bounded device-side wait (transforms, tcgen05 first or second stage) timed out");
     return RB_ERR_TIMEOUT;
   }
   if (stt.flags & RB_FLAG_CAND_OVERFLOW) {
@@ -787,7 +792,7 @@ int rb_filter(const rb_filter_desc* desc, const rb_basis* basis, const float* st
     return RB_ERR_BAD_INPUT;
   }
   if (s.flags & RB_FLAG_TIMEOUT) {
-    set_detail("a bounded device-side wait (tcgen05 first or second stage) timed out");
+    set_detail("a bounded device-side wait (transforms, tcgen05 first or second stage) timed out");
     return RB_ERR_TIMEOUT;
   }
   if ((int64_t)s.cand > desc->cand_capacity) {
@@ -961,7 +966,7 @@ int rb_filter_banks(const rb_filter_desc* descs, const rb_basis* bases, int32_t 
     return RB_ERR_BAD_INPUT;
   }
   if (s.flags & RB_FLAG_TIMEOUT) {
-    set_detail("a bounded device-side wait (tcgen05 first or second stage) timed out");
+    set_detail("a bounded device-side wait (transforms, tcgen05 first or second stage) timed out");
     return RB_ERR_TIMEOUT;
   }
   if (s.flags & RB_FLAG_CAND_OVERFLOW) {
@@ -1020,16 +1025,20 @@ static int template_first_stage(const rb_filter_desc* desc, const float* templat
   if ((rc = init_tables(f.gn, f.wn, psd, desc->fs, st))) return rc;
   if ((rc = init_tables(f.gm, f.wm, nullptr, desc->fs, st))) return rc;
   if ((rc = whiten(f.gn, f.wn, strain, f.wn.shat, st))) return rc;
-  if (!lowpass && (rc = init_gfold(f.gfold, desc->n, desc->w, st))) return rc;
+  if (!lowpass && (rc = init_gfold(f.gm, desc->n_templates, f.wn.shat, f.gfold, desc->n, desc->w, st))) return rc;
   if ((rc = folded_stage1(f.gm, f.wm, (const float2*)templates, desc->n_templates, f.wn.shat, desc->w,
-                          desc->rho_i * desc->rho_i, desc->block_id, cand, desc->cand_capacity, f.gfold, st,
-                          lowpass)))
+                          desc->rho_i * desc->rho_i, desc->block_id, cand, desc->cand_capacity, f.gfold, f.folded,
+                          f.rows, st, lowpass)))
     return rc;
   Status s;
   if ((rc = read_status(f.wn, &s, st))) return rc;
   if (s.flags & RB_FLAG_BAD_PSD) {
     set_detail("PSD not finite and positive on 0 < j < n/2");
     return RB_ERR_BAD_INPUT;
+  }
+  if (s.flags & RB_FLAG_TIMEOUT) {
+    set_detail("a bounded device-side wait of the transforms timed out");
+    return RB_ERR_TIMEOUT;
   }
   *n_cand = (int64_t)s.cand;
   if ((int64_t)s.cand > desc->cand_capacity) {
@@ -1071,6 +1080,10 @@ int rb_filter_plain(const rb_filter_desc* desc, const float* templates, const fl
   if (s.flags & RB_FLAG_BAD_PSD) {
     set_detail("PSD not finite and positive on 0 < j < n/2");
     return RB_ERR_BAD_INPUT;
+  }
+  if (s.flags & RB_FLAG_TIMEOUT) {
+    set_detail("a bounded device-side wait of the transforms timed out");
+    return RB_ERR_TIMEOUT;
   }
   *n_trig = (int64_t)s.trig;
   if ((int64_t)s.trig > capacity) {

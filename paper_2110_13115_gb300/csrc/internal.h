@@ -27,16 +27,21 @@ struct Tables {
   float2* n1_w = nullptr;    // [n1] exp(2 pi i e / n1)
   float2* n2_w = nullptr;    // [n2] exp(2 pi i e / n2)
   float2* fine_w = nullptr;  // [n2] exp(2 pi i e / n)
-  float2* w2a_w = nullptr;   // [32][n2/32 + 1]: exp(2 pi i j r / n2), stage-2 twiddles of the radix-32 pass A
-  float2* w2b_w = nullptr;   // [32][n1/32 + 1]: exp(2 pi i j r / n1), the same for pass B
+  float2* w2a_w = nullptr;   // [32][n2/32 + 1]: exp(2 pi i j r / n2), stage-2 twiddles of the fused transforms
+  float2* w4_w = nullptr;    // [n1/4]: exp(2 pi i 128 e / n), then [128]: exp(2 pi i e / n) (fused transforms)
   const float2* n1 = nullptr;
   const float2* n2 = nullptr;
   const float2* fine = nullptr;
   const float2* w2a = nullptr;
-  const float2* w2b = nullptr;
+  const float2* w4 = nullptr;
 };
 // float2 entries of a stage-2 twiddle table for a column length L
 inline int64_t w2_entries(int L) { return 32 * (int64_t)(L / 32 + 1); }
+
+// Most rows of the four-step intermediate X (96 MB, which L2 keeps), and the synchronisation words of the
+// fused transforms for that many (series.cuh: four, then two per row of the next power of two).
+inline int64_t max_x_rows(int64_t n) { return n < (int64_t(12) << 20) ? (int64_t(12) << 20) / n : 1; }
+inline int sync_words(int64_t n) { return (int)(4 + 4 * max_x_rows(n)); }
 
 // A bucketed second-stage record: the template row and block id of a run of candidates in one
 // group of bins, and the mask of those bins within the group (bit j: bin j of the group); the group
@@ -59,6 +64,7 @@ struct Workspace {
   float2* shat = nullptr;     // [n/2] whitened data
   rb_trigger* trig_stage = nullptr;  // device staging of the triggers for RB_MEM_HOST_TRIGGERS (at an
                                      // offset and size that depend on n only)
+  unsigned* sync = nullptr;   // [sync_words(n)] order of the fused transforms (series.cuh), zero between launches
   float2* X = nullptr;        // [vc][n1][n2] four-step intermediate
   int vc = 1;                 // vectors per four-step chunk
   float2* beta = nullptr;     // [k][n/2]
@@ -90,8 +96,8 @@ int bank_filter(const Geometry& g, const Workspace& ws, const float2* rows, int6
 int plain_filter(const Geometry& g, const Workspace& ws, const float2* tmpl, int64_t T, const float2* shat,
                  int w, float thr2, int64_t sample_offset, int block_id, rb_trigger* trig, int64_t cap,
                  cudaStream_t st);
-// Whether the radix-32 four-step passes run where they apply (host hook rbx_set_fft_radix32).
-bool fft_radix32_enabled();
+// Whether the fused transforms run where they apply (host hook rbx_set_fft_radix32).
+bool fft_fused_enabled();
 // FFT schedule variants of the basis filter and the template-method comparator (per n and w)
 int set_fft_variant(const Geometry& g, int w, int variant);
 int tune_fft(const Geometry& g, const Workspace& ws, const float2* rows, int64_t nvec, const float2* shat,
@@ -99,11 +105,12 @@ int tune_fft(const Geometry& g, const Workspace& ws, const float2* rows, int64_t
 // Fast first stage by the template method (Sec. III.D): gfold[j] = G(j) / w on j < n/2, then per template
 // the folded spectrum's inverse transform of length gm.n = n / w, candidates where |<z>_b|^2 >= thr2
 // (counted at wm.cand_count, at most cap stored).
-int init_gfold(float2* gfold, int64_t n, int w, cudaStream_t st);
+int init_gfold(const Geometry& gm, int64_t T, const float2* shat, float2* gfold, int64_t n, int w, cudaStream_t st);
+// folded: room for `rows` folded spectra (fused transforms, where gfold holds the weights times s_hat).
 // lowpass: the first stage of Sec. III.G instead (the product's lowest n / w bins, no fold).
 int folded_stage1(const Geometry& gm, const Workspace& wm, const float2* tmpl, int64_t T, const float2* shat, int w,
-                  float thr2, int block_id, rb_candidate* cand, int64_t cap, const float2* gfold, cudaStream_t st,
-                  bool lowpass = false);
+                  float thr2, int block_id, rb_candidate* cand, int64_t cap, const float2* gfold, float2* folded, int rows,
+                  cudaStream_t st, bool lowpass = false);
 int stage1_simt(const rb_filter_desc& d, const rb_basis& b, const Geometry& g, const Workspace& ws,
                 const float2* bavg, rb_candidate* cand, cudaStream_t st);
 int pack_beta(const rb_filter_desc& d, const Geometry& g, const float2* bavg, void* hi, void* lo,

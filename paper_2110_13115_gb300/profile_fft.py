@@ -1,10 +1,9 @@
-"""Timing driver of the basis filter's four-step passes, for profiling them one at a time.
+"""Timing driver of the basis filter's transforms, for profiling them one at a time.
 
 ``python -m paper_2110_13115_gb300.profile_fft [mode]`` filters one n = 2^19 block (w = 8) with 64
 unit-norm random basis vectors through rb_basis_filter, two warm-up calls then five timed ones, and
-the same vectors as templates through rb_filter_plain; mode 0 selects the radix-16 passes, 1 + v the
-radix-32 passes in variant v (bit 0: running-product twiddles, bit 1: pass A's rows staged in shared
-memory); "all" runs modes 4, 3, 2, 1 and 0. Prints microseconds per vector for each mode.
+the same vectors as templates through rb_filter_plain; mode 0 selects the radix-16 passes, 1 the fused
+launch (the default); "all" runs both. Prints microseconds per vector for each mode.
 """
 from __future__ import annotations
 
@@ -29,7 +28,7 @@ def main(argv):
     ws = api.workspace(d)
     sh = api.rb_whiten(d, x, psd_d, ws=ws)
     arg = argv[1] if len(argv) > 1 else "all"
-    modes = (4, 3, 2, 1, 0) if arg == "all" else (int(arg),)
+    modes = (1, 0) if arg == "all" else (int(arg),)
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     dp = api.make_desc(g.fs, n, 1, k, w=w, rho_ii=6.0)
     wsp = api.workspace(dp)
@@ -50,7 +49,7 @@ def main(argv):
                 torch.cuda.synchronize()
                 print(f"mode {mode}: {e0.elapsed_time(e1) / 5 / k * 1e3:.2f} us per {what}", flush=True)
     finally:
-        lib.rbx_set_fft_radix32(4)
+        lib.rbx_set_fft_radix32(1)
 
 
 if __name__ == "__main__":
