@@ -723,10 +723,9 @@ int rb_stage2(const rb_filter_desc* desc, const rb_basis* basis, const float* be
     return RB_ERR_BAD_INPUT;
   }
   if (n_cand > 0) {
-    const unsigned long long cnt = (unsigned long long)n_cand;
-    RB_CUDA_TRY(cudaMemcpyAsync(ws.cand, cand, sizeof(rb_candidate) * n_cand, cudaMemcpyDeviceToDevice, st));
-    RB_CUDA_TRY(cudaMemcpyAsync(ws.cand_count, &cnt, sizeof(cnt), cudaMemcpyHostToDevice, st));
-    RB_CUDA_TRY(cudaStreamSynchronize(st));  // cnt lives on this stack frame
+    // the list is read where it lies: no copy, and its length goes in with a launch instead of a synchronised copy
+    ws.cand = const_cast<rb_candidate*>(cand);
+    if ((rc = stage2_count(ws, n_cand, st))) return rc;
     if ((rc = stage2_bucketed(*desc, *basis, g, ws, (const float2*)beta, trig, capacity, ws.trig_count, 0, st))) return rc;
   }
   Status s;

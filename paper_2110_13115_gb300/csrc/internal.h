@@ -139,6 +139,8 @@ int stage2_tc_samples(const rb_filter_desc& d);
 // Bins per group for desc: stage2_tc_samples / w for the tcgen05 second stage, 1 for the mma.sync
 // one; the bucketing and the reconstruction of one call see the same value.
 int stage2_group(const rb_filter_desc& d);
+// Sets the number of candidates at ws.cand_count.
+int stage2_count(const Workspace& ws, int64_t n_cand, cudaStream_t st);
 // The two halves of stage2_bucketed: bucketing of ws.cand by bin group, then the reconstruction.
 int stage2_bucket(const rb_filter_desc& d, const Geometry& g, const Workspace& ws, int bin_lo, cudaStream_t st);
 // tmpl_base is added to every trigger's template row (sub-banks filtered into one list).

@@ -119,6 +119,8 @@ __global__ void __launch_bounds__(256) k_bin_count(const rb_candidate* __restric
   }
 }
 
+__global__ void k_set_count(unsigned long long* count, unsigned long long n) { *count = n; }
+
 constexpr int kScanPer = 16;                 // counters per thread and tile
 constexpr int kScanTile = 1024 * kScanPer;   // bins per tile (one tile for 2^19-sample blocks at w = 8)
 // one padding word per kScanPer: each thread's run of kScanPer counters starts in its own bank
@@ -578,6 +580,12 @@ namespace rb {
 int stage2_group(const rb_filter_desc& d) {
   const int samples = stage2_use_tc() ? stage2_tc_samples(d) : 0;
   return samples > 0 ? samples / d.w : 1;
+}
+
+int stage2_count(const Workspace& ws, int64_t n_cand, cudaStream_t st) {
+  k_set_count<<<1, 1, 0, st>>>(ws.cand_count, (unsigned long long)n_cand);
+  RB_LAUNCH_CHECK();
+  return RB_OK;
 }
 
 int stage2_bucket(const rb_filter_desc& d, const Geometry& g, const Workspace& ws, int bin_lo, cudaStream_t st) {
