@@ -21,7 +21,8 @@
 // they wait for: of 3.15 us a row the loads were 0.4 us and the butterflies 0.7 us. Running three items of an SM in
 // step, so that they fetch it together, brought the fetch stalls from 2.9 to 0.4 cycles per instruction and as much
 // waiting for each other's shared-memory and FP32 phases (3.27 us); two CTAs with 255 registers and a separate
-// exchange buffer: 3.2 us; L2 residency hints on X: no change; fewer instructions (no spare cases): 2.75 us.
+// exchange buffer: 3.2 us; L2 residency hints on X: no change; fewer instructions (no spare cases): 2.75 us, and with
+// short copy loops 2.71 us.
 //
 // Order and dependencies. Tickets are taken in increasing order by CTAs that are running, a CTA never
 // waits while it holds results that it has not announced, and an item depends on items of lower tickets
@@ -266,7 +267,7 @@ __global__ void __launch_bounds__(32 * WARPS, WARPS == 4 ? 3 : 1) k_series(const
     }
     return true;
   };
-  // (every thread) the tile of ticket t into shared memory
+  // (every thread) the tile of ticket t into shared memory; short loops, for the code's sake (2.76 -> 2.71 us a row)
   auto request = [&](unsigned t) {
     unsigned item;
     const int part = part_of(t, items, (unsigned)a.lag, &item);
@@ -275,29 +276,27 @@ __global__ void __launch_bounds__(32 * WARPS, WARPS == 4 ? 3 : 1) k_series(const
     const uint32_t tile_s = (uint32_t)__cvta_generic_to_shared(tile);
     if (part == 0) {
       constexpr int U = S::U;
+      // a thread's rows lie NT / U apart, a multiple of the swizzle's period, so one offset serves them all
+      static_assert((NT / U) % (SA == 4 ? 4 : 8) == 0, "swizzle period");
+      const uint32_t dst0 = tile_s + (tid / U * U + (tid % U ^ S::swz(tid / U))) * 16;
       if constexpr (FULL) {
         const float2* src = a.rows + (int64_t)vec * N + grp * S::CA + (int64_t)(tid / U) * N1 + 2 * (tid % U);
-#pragma unroll
-        for (int i = 0; i < TP / 2 / NT; ++i) {
-          const int row = tid / U + i * (NT / U);
-          cp16(tile_s + (row * U + (tid % U ^ S::swz(row))) * 16, src + (int64_t)i * (NT / U) * N1);
-        }
+#pragma unroll 4
+        for (int i = 0; i < TP / 2 / NT; ++i) cp16(dst0 + i * NT * 16, src + (int64_t)i * (NT / U) * N1);
       } else {
         const float2* src = a.rows + (int64_t)vec * HALF + grp * S::CA + (int64_t)(tid / U) * N1 + 2 * (tid % U);
         const float2* sh = a.shat + grp * S::CA + (int64_t)(tid / U) * N1 + 2 * (tid % U);
         if (a.align_rows) {
-#pragma unroll
+#pragma unroll 4
           for (int i = 0; i < TP / 4 / NT; ++i) {
-            const int row = tid / U + i * (NT / U);
-            const uint32_t dst = tile_s + (row * U + (tid % U ^ S::swz(row))) * 16;
+            const uint32_t dst = dst0 + i * NT * 16;
             cp16(dst, src + (int64_t)i * (NT / U) * N1);
             cp16(dst + TP * 4, sh + (int64_t)i * (NT / U) * N1);
           }
         } else {
 #pragma unroll 1
           for (int i = 0; i < TP / 4 / NT; ++i) {
-            const int row = tid / U + i * (NT / U);
-            const uint32_t dst = tile_s + (row * U + (tid % U ^ S::swz(row))) * 16;
+            const uint32_t dst = dst0 + i * NT * 16;
             const float2 *p = src + (int64_t)i * (NT / U) * N1, *q = sh + (int64_t)i * (NT / U) * N1;
             cp8(dst, p);
             cp8(dst + 8, p + 1);
@@ -309,7 +308,7 @@ __global__ void __launch_bounds__(32 * WARPS, WARPS == 4 ? 3 : 1) k_series(const
     } else {
       constexpr int U = S::kPairsB;
       const float2* src = a.X + (int64_t)(vec & slot_mask) * N + grp * S::CB + (int64_t)(tid / U) * N2 + 2 * (tid % U);
-#pragma unroll
+#pragma unroll 4
       for (int i = 0; i < TP / 2 / NT; ++i) cp16(tile_s + (tid + i * NT) * 16, src + (int64_t)i * (NT / U) * N2);
     }
   };
@@ -395,16 +394,25 @@ __global__ void __launch_bounds__(32 * WARPS, WARPS == 4 ? 3 : 1) k_series(const
       __syncthreads();  // the tile has been read
       dftp<32, 1, !FULL, false>(v, y);
       // exchange within the warp: y1[32 tj + k] out, y1[j + 32 r] in
+      // (eight addresses, one per low part of the point's number, and constant offsets from them)
       ulonglong2* const ex = reinterpret_cast<ulonglong2*>(tile) + pr * N2;
 #pragma unroll
-      for (int k2 = 0; k2 < 32; ++k2) ex[32 * tj + (k2 ^ (tj & 7))] = make_ulonglong2(y[k2].re, y[k2].im);
+      for (int m = 0; m < 8; ++m) {
+        ulonglong2* const e = ex + 32 * tj + (m ^ (tj & 7));
+#pragma unroll
+        for (int k2 = m; k2 < 32; k2 += 8) e[k2 - m] = make_ulonglong2(y[k2].re, y[k2].im);
+      }
       __syncwarp();
 #pragma unroll
       for (int b = 0; b < 32 / SA; ++b)
 #pragma unroll
-        for (int r = 0; r < SA; ++r) {
-          const ulonglong2 x = ex[32 * r + ((tj + SA * b) ^ (r & 7))];
-          v[b * SA + r] = {x.x, x.y};
+        for (int m = 0; m < (SA < 8 ? SA : 8); ++m) {
+          const ulonglong2* const e = ex + ((tj + SA * b) ^ m);
+#pragma unroll
+          for (int r = m; r < SA; r += 8) {
+            const ulonglong2 x = e[32 * r];
+            v[b * SA + r] = {x.x, x.y};
+          }
         }
       advance();
       // four-step twiddles w_n^(j1 (j + 32 k)), j = tj + SA b: w_n^(j1 tj) (w_n^(SA j1))^b (w_n^(32 j1))^k
