@@ -13,10 +13,17 @@
 // amp s_hat e^(i Psi), and its sums. The derivatives of Psi are linear in f, F5 = (pi f)^(-5/3), F3 = (pi f)^(-1) and
 // F2 = (pi f)^(-2/3) with coefficients that are constant over the points, so a pass sums the terms and their moments
 // with those four, and one thread forms the gradient.
-// Measured (FP64 issue bounds it, 16 operations a point): 512 candidates x 20 steps at n = 2^17 3.35 ms against
-// 17.8 ms with every point in FP64; value and gradient of 500 candidates at n = 2^19 1.61 ms against 5.11 ms. A phase in
-// pairs too would take 1.45 ms and 0.65 ms and is as accurate, but it rounds to another FP32 phase at one
-// point in some thousands, which the ascent amplifies to 1e-8 of J against the FP64 phase.
+// Measured (FP64 issue bounds it, 16 operations a point): value and gradient of 500 candidates at n = 2^19 1.48 ms
+// against 4.39 ms with every point in FP64. A phase in pairs too would take 0.65 ms and is as accurate, but it rounds to
+// another FP32 phase at one point in some thousands.
+//
+// The ascent stays in FP64 (k_refine_ascend): a last digit of the gradient is a last digit of theta, which moves the FP32
+// phase of a few points, and so J by 1e-9, and now and then the choice of a step; with pairs, J came out up to 6e-9 (norm
+// over the candidates) from what this library gave before. It does the same roundings in the same order (the FMAs
+// are written out, so that no compiler regroups them) in 45 FP64 operations a point instead of about 90: quotients by
+// reciprocals formed once per pass, 1 / v as above, tables, sine and cosine widened by their bits, no sums twice.
+// 512 candidates x 20 steps at n = 2^17: 7.11 ms against 15.3 ms, bit for bit.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -25,6 +32,8 @@
 #include "common.cuh"
 #include "internal.h"
 
+namespace cg = cooperative_groups;
+
 namespace {
 
 constexpr double kMsunS = 4.925491025543576e-06;
@@ -32,8 +41,13 @@ constexpr double kPi = 3.14159265358979323846;
 constexpr double kFref = 100.0;
 constexpr double kEtaMin = 0.05;
 constexpr int kThreads = 128;
+constexpr int kAscThreads = 256;  // threads of a candidate in the ascent
+// CTAs (a cluster) that these are spread over, in 20 steps of 512 candidates at n = 2^17 / of 64 at n = 2^15:
+// one 7.07 / 0.89 ms (two resident per SM, so that 512 leave the second wave two thirds empty), two 6.38 / 0.67,
+// four 6.81 / 0.66, eight 7.40 / 0.68.
+constexpr int kAscRanks = 2;
 
-enum { R_EVAL = 0, R_ADJOINT = 1, R_ASCEND = 2 };
+enum { R_EVAL = 0, R_ADJOINT = 1 };
 
 // Workspace header: flags, the smallest PSD value of the band (complemented bits, so that zero is "none"),
 // the first frequency above every candidate's support.
@@ -53,6 +67,9 @@ struct RefArgs {
   float2* g2;     // (F2 hi, F2 lo)
   double* amp2;   // amp^2, zero below the band
   double* chunk;  // sums of amp2 over blocks of kThreads frequencies
+  // the ascent's tables, in the place of w and amp2: s_hat and f^(-7/6) sqrt(4 df / S) in FP64
+  double2* sh;
+  double* amp;
   int64_t half, jlo;
   double df;
   double p53, p23;  // pi^(-5/3), pi^(-2/3)
@@ -195,6 +212,19 @@ __global__ void __launch_bounds__(kThreads) k_refine_tables(RefArgs a) {
   }
 }
 
+// The ascent's tables on [jlo, jmax).
+__global__ void __launch_bounds__(kThreads) k_ascend_tables(RefArgs a) {
+  const int64_t jmax = min((int64_t)a.head->jmax, a.half);
+  for (int64_t j = a.jlo + blockIdx.x * (int64_t)kThreads + threadIdx.x; j < jmax; j += (int64_t)gridDim.x * kThreads) {
+    const double f = j * a.df, vf = cbrt(kPi * f);
+    const float2 sh = a.shat[j];
+    a.v[j] = make_double2(vf, 1.0 / vf);
+    a.x[j] = 2.0 * kPi * f;
+    a.sh[j] = make_double2(sh.x, sh.y);
+    a.amp[j] = pow(f, -7.0 / 6.0) * sqrt(4.0 * a.df / a.psd[j]);
+  }
+}
+
 // --- one pass over the frequencies ---------------------------------------------------------------
 // A candidate's constants (from one thread, by way of shared memory).
 struct Point {
@@ -268,8 +298,13 @@ __device__ void evaluate(const RefArgs& a, const Point* shared, int64_t jhi, dou
     const double vv = m13 * vt.x, guess = r13 * vt.y;  // 1 / vv within two units in the last place
     const double iv = fma(guess, fma(-vv, guess, 1.0), guess);
     const double iv2 = iv * iv, iv3 = iv2 * iv, iv5 = iv3 * iv2;
-    const double psi_pn = PN3 ? c0 * (iv5 + c2 * iv3 + c3 * iv2) : c0 * (iv5 + c2 * iv3);
-    double phase = __ldg(a.x + j) * tc - phic - 0.25 * kPi + psi_pn;
+    double phase = __ldg(a.x + j) * tc - phic - 0.25 * kPi;
+    if constexpr (GRAD) {  // (rounded as in the ascent)
+      const double in = __fma_rn(c2, iv3, iv5);
+      phase = __dadd_rn(phase, __dmul_rn(c0, PN3 ? __fma_rn(c3, iv2, in) : in));
+    } else {
+      phase += PN3 ? c0 * (iv5 + c2 * iv3 + c3 * iv2) : c0 * (iv5 + c2 * iv3);
+    }
     // the nearest whole number of turns, by an addition that leaves no fraction bits (|turns| < 2^51)
     const double k = fma(phase, 1.0 / (2.0 * kPi), 6755399441055744.0) - 6755399441055744.0;
     phase -= 2.0 * kPi * k;
@@ -365,7 +400,6 @@ __global__ void __launch_bounds__(kThreads, 4) k_refine(RefArgs a) {
   __shared__ double red[(kThreads / 32) * 10];
   __shared__ Point point;
   __shared__ int64_t s_jhi;
-  __shared__ int s_go;
   const int64_t c = blockIdx.x;
   if (c >= a.n_cand) return;
   double th[4];
@@ -406,59 +440,206 @@ __global__ void __launch_bounds__(kThreads, 4) k_refine(RefArgs a) {
 #pragma unroll
       for (int k = 0; k < 4; ++k) a.dtheta[4 * c + k] = g * 2.0 * d[k] / sig2;
     }
-  } else {
-    const double scale[4] = {th[0], 1.0, 1.0 / kFref, 1.0};
-    double u[4], ut[4], grad[4], J = 0.0, alpha = a.alpha0;
+  }
+}
+
+// --- the ascent ------------------------------------------------------------------------------------
+// x / d by the correctly rounded r = 1 / d: the residual of the first guess is exact and its correction rounds once.
+__device__ __forceinline__ double quotient(double x, double d, double r) {
+  const double q = __dmul_rn(x, r);
+  return __fma_rn(__fma_rn(-d, q, x), r, q);
+}
+// a sine or cosine (zero, normal or NaN) in FP64 by its bits: conversions run at the FP64 rate
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  const unsigned hi = m == 0 ? 0u : m < 0x7f800000u ? (m >> 3) + 0x38000000u : 0x7ff80000u;
+  return __hiloint2double((int)((b & 0x80000000u) | hi), (int)(b << 29));
+}
+
+// A candidate's constants in the ascent, and the reciprocals of what is divided by.
+struct AscPoint {
+  double m13, r13, c0, c2, c3, tc, phic;
+  double k3, k2, c0d;  // 3 c2, 2 c3, c0 dc2
+  double dm, rdm, mt, mc, rmc, eta, reta, de;  // 128 eta mt, mt, mc, eta, -0.6 mt / eta
+};
+
+__device__ void make_point(const RefArgs& a, const double (&th)[4], AscPoint& p) {
+  const double mc = th[0], eta = th[1];
+  const double mt = mc * pow(eta, -0.6) * kMsunS;
+  const double dc2 = a.pn >= 2 ? (20.0 / 9.0) * (11.0 / 4.0) : 0.0;
+  p.m13 = cbrt(mt);
+  p.r13 = 1.0 / p.m13;
+  p.c0 = 3.0 / (128.0 * eta);
+  p.c2 = a.pn >= 2 ? (20.0 / 9.0) * (743.0 / 336.0 + 11.0 * eta / 4.0) : 0.0;
+  p.c3 = a.pn >= 3 ? -16.0 * kPi : 0.0;
+  p.tc = th[2];
+  p.phic = th[3];
+  p.k3 = 3.0 * p.c2;
+  p.k2 = 2.0 * p.c3;
+  p.c0d = p.c0 * dc2;
+  p.dm = 128.0 * eta * mt;
+  p.rdm = 1.0 / p.dm;
+  p.mt = mt;
+  p.mc = mc;
+  p.rmc = 1.0 / mc;
+  p.eta = eta;
+  p.reta = 1.0 / eta;
+  p.de = -0.6 * mt / eta;
+}
+
+// Z (v[0..1]) and dZ/dtheta_k (v[2 + 2k .. 3 + 2k]), on the cluster's first thread.
+template <bool PN3>
+__device__ void evaluate_fp64(const RefArgs& a, const cg::cluster_group& cluster, const AscPoint* first, int64_t jhi, double* sums,
+                              double (&v)[10]) {
+  const double m13 = first->m13, r13 = first->r13, c0 = first->c0, c2 = first->c2, c3 = first->c3, tc = first->tc, phic = first->phic;
+  const double k3 = first->k3, k2 = first->k2, c0d = first->c0d, dm = first->dm, rdm = first->rdm, mt = first->mt, mc = first->mc,
+               rmc = first->rmc, eta = first->eta, reta = first->reta, de = first->de;
+  const int tid = (int)cluster.thread_rank();
 #pragma unroll
-    for (int k = 0; k < 4; ++k) u[k] = th[k] / scale[k];
-    for (int step = -1; step < a.steps; ++step) {  // step -1: the starting point
-      if (step >= 0) {
-        if (threadIdx.x == 0) {
-          double gu[4], nrm = 0.0;
+  for (int i = 0; i < 10; ++i) v[i] = 0.0;
+  for (int64_t j = a.jlo + tid; j < jhi; j += kAscThreads) {
+    const double2 vt = __ldg(a.v + j), sh = __ldg(a.sh + j);
+    const double x = __ldg(a.x + j), am = __ldg(a.amp + j);
+    const double vv = __dmul_rn(m13, vt.x), guess = r13 * vt.y;  // 1 / vv within two units in the last place
+    const double iv = __fma_rn(guess, __fma_rn(-vv, guess, 1.0), guess);
+    const double iv2 = __dmul_rn(iv, iv), iv3 = __dmul_rn(iv2, iv), iv5 = __dmul_rn(iv3, iv2);
+    double in = __fma_rn(c2, iv3, iv5);
+    if (PN3) in = __fma_rn(c3, iv2, in);
+    const double psi_pn = __dmul_rn(c0, in);
+    double psi = __dadd_rn(__fma_rn(x, tc, -phic), -0.25 * kPi);
+    psi = __dadd_rn(psi, psi_pn);
+    const double k = __dadd_rn(__fma_rn(psi, 1.0 / (2.0 * kPi), 6755399441055744.0), -6755399441055744.0);
+    psi = __fma_rn(-2.0 * kPi, k, psi);
+    float snf, csf;
+    sincosf((float)psi, &snf, &csf);
+    const double sn = widen(snf), cs = widen(csf);
+    const double ir = __fma_rn(sh.x, cs, -__dmul_rn(sh.y, sn)), ii = __fma_rn(sh.x, sn, __dmul_rn(sh.y, cs));
+    const double tr = __dmul_rn(am, ir), ti = __dmul_rn(am, ii);
+    v[0] = __dadd_rn(v[0], tr);
+    v[1] = __dadd_rn(v[1], ti);
+    double num = __fma_rn(-5.0, iv5, -__dmul_rn(k3, iv3));
+    if (PN3) num = __fma_rn(-k2, iv2, num);
+    const double dpsi = quotient(num, dm, rdm);
+    const double d0 = quotient(__dmul_rn(dpsi, mt), mc, rmc);
+    const double deta = __dadd_rn(__dmul_rn(c0d, iv3), quotient(-psi_pn, eta, reta));
+    const double d1 = __fma_rn(dpsi, de, deta);
+    v[2] = __fma_rn(-d0, ti, v[2]);
+    v[3] = __fma_rn(d0, tr, v[3]);
+    v[4] = __fma_rn(-d1, ti, v[4]);
+    v[5] = __fma_rn(d1, tr, v[5]);
+    v[6] = __fma_rn(-x, ti, v[6]);
+    v[7] = __fma_rn(x, tr, v[7]);
+  }
+  constexpr int NV = 8;
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            gu[k] = grad[k] * scale[k];
-            nrm += gu[k] * gu[k];
-          }
-          nrm = sqrt(nrm);
-          s_go = nrm > 0.0;
-          if (nrm > 0.0) {
+  for (int i = 0; i < NV; ++i)
 #pragma unroll
-            for (int k = 0; k < 4; ++k) ut[k] = u[k] + alpha * gu[k] / nrm;
-            ut[1] = fmin(fmax(ut[1], kEtaMin), 0.25);
-            double tt[4];
+    for (int off = 16; off > 0; off >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], off);
+  if ((tid & 31) == 0)
 #pragma unroll
-            for (int k = 0; k < 4; ++k) tt[k] = ut[k] * scale[k];
-            make_point(a, tt, point);
-          }
-        }
-        __syncthreads();
-        if (!s_go) break;  // (the gradient stays what it is)
-      }
-      evaluate<true, PN3>(a, &point, jhi, red, s);
-      if (threadIdx.x == 0) {
-        const double Jt = (s.z[0] * s.z[0] + s.z[1] * s.z[1]) / sig2;
-        if (step < 0 || Jt > J) {
-          J = Jt;
-          double d[4];
-          derivatives(a, point, s, s.z[0], s.z[1], d);
+    for (int i = 0; i < NV; ++i) sums[(tid >> 5) * 10 + i] = v[i];
+  cluster.sync();
+  if (tid == 0) {
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            if (step >= 0) u[k] = ut[k];
-            grad[k] = 2.0 * d[k] / sig2;
-          }
-          if (step >= 0) alpha = fmin(2.0 * alpha, a.alpha_max);
-        } else {
-          alpha *= 0.5;
-        }
-      }
+    for (int i = 0; i < NV; ++i) {
+      double s = 0.0;
+      for (int w = 0; w < kAscThreads / 32; ++w) s += sums[w * 10 + i];
+      v[i] = s;
     }
-    if (threadIdx.x == 0) {
+    v[8] = v[1];  // dPsi/dphi_c = -1
+    v[9] = -v[0];
+  }
+}
+
+template <bool PN3>
+__global__ void __launch_bounds__(kAscThreads / kAscRanks, 2 * kAscRanks) k_refine_ascend(RefArgs a) {
+  // (of the cluster's first CTA)
+  __shared__ double red[(kAscThreads / 32) * 10];
+  __shared__ AscPoint point;
+  __shared__ int64_t s_jhi;
+  __shared__ int s_go;
+  const cg::cluster_group cluster = cg::this_cluster();
+  const int tid = (int)cluster.thread_rank();
+  const int64_t c = blockIdx.x / kAscRanks;
+  const AscPoint* const first = cluster.map_shared_rank(&point, 0);
+  double* const sums = cluster.map_shared_rank(red, 0);
+  double th[4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) a.theta_out[4 * c + k] = u[k] * scale[k];
-      a.J[c] = J;
+  for (int i = 0; i < 4; ++i) th[i] = a.theta_in[4 * c + i];
+  if (!(th[0] > 0.0) || !(th[1] > 0.0) || !(th[1] <= 0.25) || !isfinite(th[2]) || !isfinite(th[3])) {
+    if (tid == 0) {
+      atomicOr(&a.head->flags, (unsigned)RB_FLAG_BAD_STRAIN);
+      a.J[c] = __longlong_as_double(0x7ff8000000000000ll);
+    }
+    return;  // (every CTA of the cluster)
+  }
+  if (tid == 0) {
+    s_jhi = support_end(a, th[0], th[1]);
+    make_point(a, th, point);
+  }
+  cluster.sync();
+  const int64_t jhi = min(*cluster.map_shared_rank(&s_jhi, 0), (int64_t)a.head->jmax);
+  double sig2 = 0.0;
+  for (int64_t j = a.jlo + tid; j < jhi; j += kAscThreads) sig2 += a.amp[j] * a.amp[j];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) sig2 += __shfl_xor_sync(0xffffffffu, sig2, off);
+  if ((tid & 31) == 0) sums[tid >> 5] = sig2;
+  cluster.sync();
+  if (tid == 0) {
+    sig2 = 0.0;
+    for (int w = 0; w < kAscThreads / 32; ++w) sig2 += red[w];
+  }
+  cluster.sync();  // (red is free again)
+  const double scale[4] = {th[0], 1.0, 1.0 / kFref, 1.0};
+  double v[10], u[4], ut[4], grad[4], J = 0.0, alpha = a.alpha0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) u[k] = th[k] / scale[k];
+  for (int step = -1; step < a.steps; ++step) {  // step -1: the starting point
+    if (step >= 0) {
+      if (tid == 0) {
+        double gu[4], nrm = 0.0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          gu[k] = grad[k] * scale[k];
+          nrm += gu[k] * gu[k];
+        }
+        nrm = sqrt(nrm);
+        s_go = nrm > 0.0;
+        if (nrm > 0.0) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) ut[k] = u[k] + alpha * gu[k] / nrm;
+          ut[1] = fmin(fmax(ut[1], kEtaMin), 0.25);
+          double tt[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) tt[k] = ut[k] * scale[k];
+          make_point(a, tt, point);
+        }
+      }
+      cluster.sync();
+      if (!*cluster.map_shared_rank(&s_go, 0)) break;  // (the gradient stays what it is)
+    }
+    evaluate_fp64<PN3>(a, cluster, first, jhi, sums, v);
+    if (tid == 0) {
+      const double Jt = (v[0] * v[0] + v[1] * v[1]) / sig2;
+      if (step < 0 || Jt > J) {
+        J = Jt;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          if (step >= 0) u[k] = ut[k];
+          grad[k] = 2.0 * __fma_rn(v[0], v[2 + 2 * k], __dmul_rn(v[1], v[3 + 2 * k])) / sig2;
+        }
+        if (step >= 0) alpha = fmin(2.0 * alpha, a.alpha_max);
+      } else {
+        alpha *= 0.5;
+      }
     }
   }
+  if (tid == 0) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) a.theta_out[4 * c + k] = u[k] * scale[k];
+    a.J[c] = J;
+  }
+  cluster.sync();  // the first CTA's shared memory is read until here
 }
 
 size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -473,17 +654,19 @@ size_t carve(int64_t half, char* base, RefArgs* a) {
   };
   a->head = (Header*)take(256);
   a->w = (float4*)take(sizeof(float4) * half);
+  a->sh = (double2*)a->w;
   a->v = (double2*)take(sizeof(double2) * half);
   a->x = (double*)take(sizeof(double) * half);
   a->g = (float4*)take(sizeof(float4) * half);
   a->g2 = (float2*)take(sizeof(float2) * half);
   a->amp2 = (double*)take(sizeof(double) * half);
+  a->amp = a->amp2;
   a->chunk = (double*)take(sizeof(double) * ((half + kThreads - 1) / kThreads));
   return off;
 }
 
 int prepare(const rb_refine_desc* d, const float* shat, const double* psd, const void* theta, int64_t n_cand,
-            void* ws, size_t bytes, RefArgs& a, cudaStream_t st) {
+            void* ws, size_t bytes, bool ascent, RefArgs& a, cudaStream_t st) {
   if (!d || !shat || !psd || !theta || n_cand < 0) {
     rb::set_detail("NULL argument or negative count");
     return RB_ERR_BAD_INPUT;
@@ -520,20 +703,17 @@ int prepare(const rb_refine_desc* d, const float* shat, const double* psd, const
   RB_CUDA_TRY(cudaMemsetAsync(a.head, 0, 256, st));
   k_refine_check<<<(int)std::min<int64_t>(304, (half + kThreads - 1) / kThreads), kThreads, 0, st>>>(a);
   RB_LAUNCH_CHECK();
-  k_refine_tables<<<(int)std::min<int64_t>(1216, (half + kThreads - 1) / kThreads), kThreads, 0, st>>>(a);
+  const int blocks = (int)std::min<int64_t>(1216, (half + kThreads - 1) / kThreads);
+  if (ascent)
+    k_ascend_tables<<<blocks, kThreads, 0, st>>>(a);
+  else
+    k_refine_tables<<<blocks, kThreads, 0, st>>>(a);
   RB_LAUNCH_CHECK();
   return RB_OK;
 }
 
-template <int MODE>
-int run(const RefArgs& a, cudaStream_t st) {
-  if (a.n_cand > 0) {
-    if (a.pn >= 3)
-      k_refine<MODE, true><<<(unsigned)a.n_cand, kThreads, 0, st>>>(a);
-    else
-      k_refine<MODE, false><<<(unsigned)a.n_cand, kThreads, 0, st>>>(a);
-    RB_LAUNCH_CHECK();
-  }
+// The call's status, once its kernels are done.
+int finish(const RefArgs& a, cudaStream_t st) {
   unsigned flags = 0;
   RB_CUDA_TRY(cudaMemcpyAsync(&flags, &a.head->flags, sizeof(flags), cudaMemcpyDeviceToHost, st));
   RB_CUDA_TRY(cudaStreamSynchronize(st));
@@ -546,6 +726,36 @@ int run(const RefArgs& a, cudaStream_t st) {
     return RB_ERR_BAD_INPUT;
   }
   return RB_OK;
+}
+
+template <int MODE>
+int run(const RefArgs& a, cudaStream_t st) {
+  if (a.n_cand > 0) {
+    if (a.pn >= 3)
+      k_refine<MODE, true><<<(unsigned)a.n_cand, kThreads, 0, st>>>(a);
+    else
+      k_refine<MODE, false><<<(unsigned)a.n_cand, kThreads, 0, st>>>(a);
+    RB_LAUNCH_CHECK();
+  }
+  return finish(a, st);
+}
+
+int ascend(const RefArgs& a, cudaStream_t st) {
+  if (a.n_cand > 0) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kAscRanks;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(a.n_cand * kAscRanks));
+    cfg.blockDim = dim3(kAscThreads / kAscRanks);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    RB_CUDA_TRY(a.pn >= 3 ? cudaLaunchKernelEx(&cfg, k_refine_ascend<true>, a) : cudaLaunchKernelEx(&cfg, k_refine_ascend<false>, a));
+    RB_LAUNCH_CHECK();
+  }
+  return finish(a, st);
 }
 
 }  // namespace
@@ -562,7 +772,7 @@ int rb_refine_eval(const rb_refine_desc* d, const float* s_hat, const double* ps
                    double* Z, int64_t n_cand, void* workspace, size_t workspace_bytes, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   RefArgs a{};
-  int rc = prepare(d, s_hat, psd, theta, n_cand, workspace, workspace_bytes, a, st);
+  int rc = prepare(d, s_hat, psd, theta, n_cand, workspace, workspace_bytes, false, a, st);
   if (rc) return rc;
   if (!J || !Z) {
     rb::set_detail("NULL output");
@@ -578,7 +788,7 @@ int rb_refine_adjoint(const rb_refine_desc* d, const float* s_hat, const double*
                       size_t workspace_bytes, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   RefArgs a{};
-  int rc = prepare(d, s_hat, psd, theta, n_cand, workspace, workspace_bytes, a, st);
+  int rc = prepare(d, s_hat, psd, theta, n_cand, workspace, workspace_bytes, false, a, st);
   if (rc) return rc;
   if (!Z || !dJ || !dtheta) {
     rb::set_detail("NULL argument");
@@ -594,7 +804,7 @@ int rb_refine(const rb_refine_desc* d, const float* s_hat, const double* psd, do
               int64_t n_cand, void* workspace, size_t workspace_bytes, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   RefArgs a{};
-  int rc = prepare(d, s_hat, psd, theta, n_cand, workspace, workspace_bytes, a, st);
+  int rc = prepare(d, s_hat, psd, theta, n_cand, workspace, workspace_bytes, true, a, st);
   if (rc) return rc;
   if (!J) {
     rb::set_detail("NULL output");
@@ -602,7 +812,7 @@ int rb_refine(const rb_refine_desc* d, const float* s_hat, const double* psd, do
   }
   a.theta_out = theta;
   a.J = J;
-  return run<R_ASCEND>(a, st);
+  return ascend(a, st);
 }
 
 }  // extern "C"
