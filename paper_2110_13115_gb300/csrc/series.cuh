@@ -14,7 +14,7 @@
 // barrier and its results leave as runs of L / 4 contiguous bytes; in part B the lanes span the columns,
 // which makes the loads, the stores of beta and the bin sums contiguous.
 //
-// What bounds it, and what was measured (n = 2^19, 201 rows, w = 8): 552 us against 892 us for two radix-32 launches
+// What bounds it, and what was measured (n = 2^19, 201 rows, w = 8): 538 us against 892 us for two radix-32 launches
 // per chunk of 8 rows, which it replaces (132 us are the rows' HBM bytes). The launches lost 512 work items to
 // 456 resident CTAs, a gap and a ramp each. Three CTAs of 128 threads fit an SM (168 registers, 74 KB); the issue
 // slots are busy 30 % of the time and the long straight-line code of an item (about 2000 instructions a warp) is what
@@ -22,7 +22,7 @@
 // step, so that they fetch it together, brought the fetch stalls from 2.9 to 0.4 cycles per instruction and as much
 // waiting for each other's shared-memory and FP32 phases (3.27 us); two CTAs with 255 registers and a separate
 // exchange buffer: 3.2 us; L2 residency hints on X: no change; fewer instructions (no spare cases): 2.75 us, and with
-// short copy loops 2.71 us.
+// short copy loops and exchange addresses 2.69 us.
 //
 // Order and dependencies. Tickets are taken in increasing order by CTAs that are running, a CTA never
 // waits while it holds results that it has not announced, and an item depends on items of lower tickets
@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(32 * WARPS, WARPS == 4 ? 3 : 1) k_series(const
     }
     return true;
   };
-  // (every thread) the tile of ticket t into shared memory; short loops, for the code's sake (2.76 -> 2.71 us a row)
+  // (every thread) the tile of ticket t into shared memory; short loops, for the code's sake (2.76 -> 2.71 us a row with them)
   auto request = [&](unsigned t) {
     unsigned item;
     const int part = part_of(t, items, (unsigned)a.lag, &item);
