@@ -2,7 +2,7 @@
 // template at its own coalescence time, its adjoint with respect to theta = (mc, eta, t_c, phi_c),
 // and an in-kernel gradient ascent. The matched filter is Eq. (1) of arXiv:2110.13115 evaluated at
 // t_0 = t_c (Eq. 3-4); the paper stops at the triggers, so the ascent rule is this library's own
-// (see include/rbmf.h). One CTA per candidate recomputes the whitened template frequency by
+// (see include/rbmf.h). One CTA or a cluster per candidate recomputes the whitened template frequency by
 // frequency in every pass.
 //
 // Arithmetic. The GPU does two FP64 operations per clock and SM against 128 in FP32, and a point took about 90 of
@@ -41,6 +41,7 @@ constexpr double kPi = 3.14159265358979323846;
 constexpr double kFref = 100.0;
 constexpr double kEtaMin = 0.05;
 constexpr int kThreads = 128;
+constexpr int kMaxRanks = 8;  // CTAs (a cluster) that share a candidate's frequencies in value and adjoint, at most
 constexpr int kAscThreads = 256;  // threads of a candidate in the ascent
 // CTAs (a cluster) that these are spread over, in 20 steps of 512 candidates at n = 2^17 / of 64 at n = 2^15:
 // one 7.07 / 0.89 ms (two resident per SM, so that 512 leave the second wave two thirds empty), two 6.38 / 0.67,
@@ -255,7 +256,7 @@ __device__ void make_point(const RefArgs& a, const double (&th)[4], Point& p) {
   p.e2 = -0.6 * a2 / eta;
 }
 
-// The sums of a pass (thread 0 after evaluate): Z and the moments with j, F5, F3, F2.
+// The sums of a pass (thread 0 of the cluster's first CTA after evaluate): Z and the moments with j, F5, F3, F2.
 struct Sums {
   double z[2], s1[2], m5[2], m3[2], m2[2];
 };
@@ -285,14 +286,17 @@ __device__ __forceinline__ void warp_sums(Sum (&v)[V], double* out) {
   if ((lane & (kCopies - 1)) == 0) out[first] = (double)v[0].h + ((double)v[0].m + (double)v[0].l);
 }
 
+// `first` and `parts` lie in the shared memory of the cluster's first CTA: the constants, and the CTAs' partial sums.
 template <bool GRAD, bool PN3>
-__device__ void evaluate(const RefArgs& a, const Point* shared, int64_t jhi, double* red, Sums& out) {
+__device__ void evaluate(const RefArgs& a, const cg::cluster_group& cluster, const Point* first, int64_t jhi, double* red,
+                         double* parts, Sums& out) {
   constexpr int V = GRAD ? 8 : 2;
-  const double m13 = shared->m13, r13 = shared->r13, c0 = shared->c0, c2 = shared->c2, c3 = shared->c3, tc = shared->tc,
-               phic = shared->phic;
+  const int rank = (int)cluster.block_rank(), ranks = (int)cluster.num_blocks();
+  const double m13 = first->m13, r13 = first->r13, c0 = first->c0, c2 = first->c2, c3 = first->c3, tc = first->tc,
+               phic = first->phic;
   Sum v[V] = {}, v2[2] = {};
 #pragma unroll 2
-  for (int64_t j = a.jlo + threadIdx.x; j < jhi; j += kThreads) {
+  for (int64_t j = a.jlo + rank * kThreads + threadIdx.x; j < jhi; j += ranks * kThreads) {
     const float4 w = __ldg(a.w + j);
     const double2 vt = __ldg(a.v + j);
     const double vv = m13 * vt.x, guess = r13 * vt.y;  // 1 / vv within two units in the last place
@@ -345,7 +349,7 @@ __device__ void evaluate(const RefArgs& a, const Point* shared, int64_t jhi, dou
       }
     }
   }
-  // block sums: pairs within a warp, FP64 across the warps
+  // sums over a warp in parts, over the warps and the cluster's CTAs in FP64
   constexpr int NV = GRAD && PN3 ? V + 2 : V;
   __syncthreads();  // (red may still be read from the pass before)
   warp_sums<V>(v, red + (threadIdx.x >> 5) * NV);
@@ -354,7 +358,14 @@ __device__ void evaluate(const RefArgs& a, const Point* shared, int64_t jhi, dou
   if (threadIdx.x < NV) {
     double t = red[threadIdx.x];
     for (int k = 1; k < kThreads / 32; ++k) t += red[k * NV + threadIdx.x];
-    red[threadIdx.x] = t;  // (only this thread reads this column)
+    parts[rank * 10 + threadIdx.x] = t;
+  }
+  cluster.sync();
+  if (rank != 0) return;
+  if (threadIdx.x < NV) {
+    double t = parts[threadIdx.x];
+    for (int k = 1; k < ranks; ++k) t += parts[k * 10 + threadIdx.x];
+    red[threadIdx.x] = t;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -397,43 +408,49 @@ __device__ __forceinline__ int64_t support_end(const RefArgs& a, double mc0, dou
 
 template <int MODE, bool PN3>
 __global__ void __launch_bounds__(kThreads, 4) k_refine(RefArgs a) {
-  __shared__ double red[(kThreads / 32) * 10];
+  // (of the cluster's first CTA: point, parts, s_jhi)
+  __shared__ double red[(kThreads / 32) * 10], parts[kMaxRanks * 10];
   __shared__ Point point;
   __shared__ int64_t s_jhi;
-  const int64_t c = blockIdx.x;
-  if (c >= a.n_cand) return;
+  const cg::cluster_group cluster = cg::this_cluster();
+  const bool lead = cluster.block_rank() == 0;
+  const int64_t c = blockIdx.x / cluster.num_blocks();
+  const Point* const first = cluster.map_shared_rank(&point, 0);
+  double* const sums = cluster.map_shared_rank(parts, 0);
   double th[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) th[i] = a.theta_in[4 * c + i];
   if (!(th[0] > 0.0) || !(th[1] > 0.0) || !(th[1] <= 0.25) || !isfinite(th[2]) || !isfinite(th[3])) {
-    if (threadIdx.x == 0) {
+    if (lead && threadIdx.x == 0) {
       atomicOr(&a.head->flags, (unsigned)RB_FLAG_BAD_STRAIN);
       if (a.J) a.J[c] = __longlong_as_double(0x7ff8000000000000ll);
     }
-    return;
+    return;  // (every CTA of the cluster)
   }
-  if (threadIdx.x == 0) s_jhi = support_end(a, th[0], th[1]);
-  if (threadIdx.x == 32) make_point(a, th, point);
-  __syncthreads();
-  const int64_t jhi = min(s_jhi, (int64_t)a.head->jmax);
+  if (lead && threadIdx.x == 0) s_jhi = support_end(a, th[0], th[1]);
+  if (lead && threadIdx.x == 32) make_point(a, th, point);
+  cluster.sync();
+  const int64_t jhi = min(*cluster.map_shared_rank(&s_jhi, 0), (int64_t)a.head->jmax);
   // sigma^2 from the chunk sums and the last chunk's part
-  double s2 = 0.0;
-  const int64_t whole = jhi / kThreads;
-  for (int64_t k = a.jlo / kThreads + threadIdx.x; k < whole; k += kThreads) s2 += a.chunk[k];
-  if (whole * kThreads + threadIdx.x < jhi && whole * kThreads + threadIdx.x >= a.jlo) s2 += a.amp2[whole * kThreads + threadIdx.x];
-  const double sig2 = block_sum(s2, red);  // (thread 0)
+  double sig2 = 0.0;  // (the lead's thread 0)
+  if (lead) {
+    const int64_t whole = jhi / kThreads, part = whole * kThreads + threadIdx.x;
+    for (int64_t k = a.jlo / kThreads + threadIdx.x; k < whole; k += kThreads) sig2 += a.chunk[k];
+    if (part < jhi && part >= a.jlo) sig2 += a.amp2[part];
+    sig2 = block_sum(sig2, red);
+  }
   Sums s;
   if (MODE == R_EVAL) {
-    evaluate<false, PN3>(a, &point, jhi, red, s);
-    if (threadIdx.x == 0) {
+    evaluate<false, PN3>(a, cluster, first, jhi, red, sums, s);
+    if (lead && threadIdx.x == 0) {
       const double unit = scalbn(1.0, -amp_scale(a));
       a.J[c] = (s.z[0] * s.z[0] + s.z[1] * s.z[1]) / sig2;
       a.Z[2 * c] = s.z[0] * unit;
       a.Z[2 * c + 1] = s.z[1] * unit;
     }
   } else if (MODE == R_ADJOINT) {
-    evaluate<true, PN3>(a, &point, jhi, red, s);
-    if (threadIdx.x == 0) {
+    evaluate<true, PN3>(a, cluster, first, jhi, red, sums, s);
+    if (lead && threadIdx.x == 0) {
       const double unit = scalbn(1.0, amp_scale(a)), g = a.dJ[c];
       double d[4];
       derivatives(a, point, s, a.Z[2 * c] * unit, a.Z[2 * c + 1] * unit, d);
@@ -731,10 +748,24 @@ int finish(const RefArgs& a, cudaStream_t st) {
 template <int MODE>
 int run(const RefArgs& a, cudaStream_t st) {
   if (a.n_cand > 0) {
-    if (a.pn >= 3)
-      k_refine<MODE, true><<<(unsigned)a.n_cand, kThreads, 0, st>>>(a);
-    else
-      k_refine<MODE, false><<<(unsigned)a.n_cand, kThreads, 0, st>>>(a);
+    // CTAs per candidate: more while the chip (152 SMs, up to four of these CTAs each) has room for them and a thread
+    // keeps 32 frequencies of the block. Value and adjoint with 1 / 2 / 4 / 8 CTAs, us: n = 2^19, 16 candidates
+    // 786 / 465 / 318 / 271, 64: 775 / 466 / 382 / 379, 128: 771 / 591 / 566 / 611, 227: 971 / 761 / 923 / 882,
+    // 456: 1318 / 1550 / 1508 / 1515; n = 2^17, 64: 303 / 224 / 207 / 220, 227: 358 / 301 / 391 / 386; n = 2^14, 64:
+    // 157 / 150 / 150 / 174, 300: 168 / 184 / 230 / 284.
+    int ranks = 1;
+    while (ranks < kMaxRanks && 2 * ranks * a.n_cand <= 512 && a.half / (2 * ranks * kThreads) >= 32) ranks *= 2;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)ranks;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(a.n_cand * ranks));
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    RB_CUDA_TRY(a.pn >= 3 ? cudaLaunchKernelEx(&cfg, k_refine<MODE, true>, a) : cudaLaunchKernelEx(&cfg, k_refine<MODE, false>, a));
     RB_LAUNCH_CHECK();
   }
   return finish(a, st);
