@@ -13,6 +13,10 @@
 // amp s_hat e^(i Psi), and its sums. The derivatives of Psi are linear in f, F5 = (pi f)^(-5/3), F3 = (pi f)^(-1) and
 // F2 = (pi f)^(-2/3) with coefficients that are constant over the points, so a pass sums the terms and their moments
 // with those four, and one thread forms the gradient.
+// Range. amp goes with the PSD and the units of the strain over hundreds of decades, s_hat over FP32's: the products
+// amp s_hat are formed in FP64 and kept as pairs of order one with an exponent of their own (four bytes a frequency),
+// and a candidate takes them relative to the largest exponent of its own support. So neither a bin outside the support
+// nor another candidate moves them, and what is lost is 2^-126 of the support's largest value and below.
 // Measured (FP64 issue bounds it, 16 operations a point): value and gradient of 500 candidates at n = 2^19 1.48 ms
 // against 4.39 ms with every point in FP64. A phase in pairs too would take 0.65 ms and is as accurate, but it rounds to
 // another FP32 phase at one point in some thousands.
@@ -50,30 +54,32 @@ constexpr int kAscRanks = 2;
 
 enum { R_EVAL = 0, R_ADJOINT = 1 };
 
-// Workspace header: flags, the smallest PSD value of the band (complemented bits, so that zero is "none"),
-// the first frequency above every candidate's support.
+// Workspace header: flags, the first frequency above every candidate's support.
 struct Header {
   unsigned flags, jmax;
-  unsigned long long smin;
 };
 
 struct RefArgs {
   const float2* shat;
   const double* psd;
   Header* head;
-  float4* w;      // amp s_hat as pairs: (re hi, im hi, re lo, im lo), amp = 2^scale f^(-7/6) sqrt(4 df / S)
+  float4* w;      // 2^-e amp s_hat as pairs: (re hi, im hi, re lo, im lo), amp = f^(-7/6) sqrt(4 df / S)
+  int* e;         // the exponent of its larger part
   double2* v;     // (vf, 1 / vf), vf = (pi f)^(1/3)
   double* x;      // 2 pi f
-  float4* g;      // (F5 hi, F5 lo, F3 hi, F3 lo)
-  float2* g2;     // (F2 hi, F2 lo)
+  float4* g;      // (F5 hi, F5 lo, F3 hi, F3 lo) over their values at the band's first frequency
+  float2* g2;     // (F2 hi, F2 lo), the same
   double* amp2;   // amp^2, zero below the band
   double* chunk;  // sums of amp2 over blocks of kThreads frequencies
+  int* top;       // the largest e of these blocks
   // the ascent's tables, in the place of w and amp2: s_hat and f^(-7/6) sqrt(4 df / S) in FP64
   double2* sh;
   double* amp;
   int64_t half, jlo;
   double df;
-  double p53, p23;  // pi^(-5/3), pi^(-2/3)
+  double amp0;                       // amp = amp0 j^(-7/6) / sqrt(S)
+  double r53, r33, r23;              // jlo^(5/3), jlo, jlo^(2/3)
+  double f5, f3, f2;                 // F5, F3, F2 at the band's first frequency
   int pn;
   const double* theta_in;
   double* theta_out;
@@ -124,24 +130,20 @@ __device__ __forceinline__ Pair mul(Pair a, float bh, float bl) {
   return {p, __fmaf_rn(a.l, bh, __fmaf_rn(a.h, bl, __fmaf_rn(a.h, bh, -p)))};
 }
 
-// The scale of the amplitudes: a power of two that brings the largest of them (at the lowest frequency and the
-// smallest PSD value, were they together) to about one, whatever the units of the strain.
-__device__ __forceinline__ int amp_scale(const RefArgs& a) {
-  const int ex = (int)((~a.head->smin >> 52) & 2047) - 1023;
-  const float flo = (float)a.jlo * (float)a.df;
-  return -(int)floorf(0.5f * (log2f(4.f * (float)a.df) - (float)ex) - 7.f / 6.f * log2f(flo)) - 1;
+// The exponent e of a complex value: its larger part lies in [2^e, 2^(e + 1)) (zero and below FP64's normal range:
+// -1023; not finite: 1024).
+__device__ __forceinline__ int exponent(double re, double im) {
+  return (int)(__double_as_longlong(fmax(fabs(re), fabs(im))) >> 52) - 1023;
 }
 
-// PSD check (0 < j < half), the band's smallest value, and the end of the candidates' supports (an FP32
-// estimate with a margin: it only bounds the tables).
+// PSD check (0 < j < half), and the end of the candidates' supports (an FP32 estimate with a margin: it only bounds
+// the tables).
 __global__ void __launch_bounds__(kThreads) k_refine_check(RefArgs a) {
   const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
-  unsigned long long low = 0;
   bool bad = false;
   for (int64_t j = tid + 1; j < a.half; j += stride) {
     const double S = a.psd[j];
     if (!(S > 0.0) || isinf(S)) bad = true;
-    else if (j >= a.jlo) low = max(low, ~(unsigned long long)__double_as_longlong(S));
   }
   unsigned top = 0;
   for (int64_t c = tid; c < a.n_cand; c += stride) {
@@ -153,13 +155,9 @@ __global__ void __launch_bounds__(kThreads) k_refine_check(RefArgs a) {
     const float fcut = 1.001f / (14.6969385f * (float)kPi * mc * powf(eta, -0.6f) * (float)kMsunS);
     top = max(top, (unsigned)fminf((float)a.half, fcut / (float)a.df + 4.f));
   }
-  for (int off = 16; off > 0; off >>= 1) {
-    low = max(low, __shfl_xor_sync(0xffffffffu, low, off));
-    top = max(top, __shfl_xor_sync(0xffffffffu, top, off));
-  }
+  top = __reduce_max_sync(0xffffffffu, top);
   bad = __any_sync(0xffffffffu, bad);
   if ((threadIdx.x & 31) == 0) {
-    if (low) atomicMax(&a.head->smin, low);
     if (top) atomicMax(&a.head->jmax, top);
     if (bad) atomicOr(&a.head->flags, (unsigned)RB_FLAG_BAD_PSD);
   }
@@ -177,28 +175,45 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   return v;
 }
 
-// The tables on [jlo, jmax): everything is a power of y = f^(-1/6) (an FP32 estimate and two Newton steps in
+// The largest of one int per thread over the block (every thread calls and receives it).
+__device__ __forceinline__ int block_max(int v, int* red) {
+  v = __reduce_max_sync(0xffffffffu, v);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = red[0];
+#pragma unroll
+  for (int w = 1; w < kThreads / 32; ++w) v = max(v, red[w]);
+  return v;
+}
+
+constexpr int kNoExponent = -(1 << 20);  // of frequencies outside the band
+
+// The tables on [jlo, jmax): everything is a power of y = j^(-1/6) (an FP32 estimate and two Newton steps in
 // FP64: the error 3.5 e^2 of a step takes 1e-6 below the rounding of FP64).
 __global__ void __launch_bounds__(kThreads) k_refine_tables(RefArgs a) {
   __shared__ double red[kThreads / 32];
+  __shared__ int red_e[kThreads / 32];
   const int64_t jmax = min((int64_t)a.head->jmax, a.half);
-  const double scale = scalbn(2.0 * sqrt(a.df), amp_scale(a));
   for (int64_t c = a.jlo / kThreads + blockIdx.x; c * kThreads < jmax; c += gridDim.x) {
     const int64_t j = c * kThreads + threadIdx.x;
     double a2 = 0.0;
+    int e = kNoExponent;
     if (j >= a.jlo && j < jmax) {
-      const double f = j * a.df;
-      double y = (double)exp2f(log2f((float)f) * (-1.f / 6.f));
+      const double f = j * a.df, x = (double)(int)j;
+      double y = (double)exp2f(log2f((float)(int)j) * (-1.f / 6.f));
 #pragma unroll
       for (int it = 0; it < 2; ++it) {
         const double y2 = y * y, y6 = y2 * y2 * y2;
-        y = y * (fma(-f, y6, 7.0) * (1.0 / 6.0));
+        y = y * (fma(-x, y6, 7.0) * (1.0 / 6.0));
       }
       const double y2 = y * y, y4 = y2 * y2, y6 = y4 * y2, y10 = y6 * y4;
-      const double am = scale * (y6 * y) * rsqrt(a.psd[j]);
+      const double am = a.amp0 * (y6 * y) * rsqrt(a.psd[j]);
       const float2 sh = a.shat[j];
-      const Pair re = to_pair(am * (double)sh.x), im = to_pair(am * (double)sh.y);
-      const Pair f5 = to_pair(a.p53 * y10), f3 = to_pair(y6 * (1.0 / kPi)), f2 = to_pair(a.p23 * y4);
+      const double wr = am * (double)sh.x, wi = am * (double)sh.y;
+      e = exponent(wr, wi);
+      const Pair re = to_pair(scalbn(wr, -e)), im = to_pair(scalbn(wi, -e));
+      const Pair f5 = to_pair(a.r53 * y10), f3 = to_pair(a.r33 * y6), f2 = to_pair(a.r23 * y4);
       const double vf = cbrt(kPi * f);
       a.v[j] = make_double2(vf, 1.0 / vf);
       a.x[j] = 2.0 * kPi * f;
@@ -207,9 +222,16 @@ __global__ void __launch_bounds__(kThreads) k_refine_tables(RefArgs a) {
       a.g2[j] = make_float2(f2.h, f2.l);
       a2 = am * am;
     }
-    if (j < a.half) a.amp2[j] = a2;
+    if (j < a.half) {
+      a.amp2[j] = a2;
+      a.e[j] = e;
+    }
     a2 = block_sum(a2, red);
-    if (threadIdx.x == 0) a.chunk[c] = a2;
+    e = block_max(e, red_e);
+    if (threadIdx.x == 0) {
+      a.chunk[c] = a2;
+      a.top[c] = e;
+    }
   }
 }
 
@@ -247,12 +269,13 @@ __device__ void make_point(const RefArgs& a, const double (&th)[4], Point& p) {
   p.c3 = c3;
   p.tc = tc;
   p.phic = phic;
-  // Psi = A5 F5 + A3 F3 + A2 F2
-  const double r2 = p.r13 * p.r13, a5 = p.c0 * (r2 * r2 * p.r13), a3 = p.c0 * c2 * (r2 * p.r13), a2 = p.c0 * c3 * r2;
+  // Psi = A5 F5 + A3 F3 + A2 F2, the F's over their values at the band's first frequency
+  const double r2 = p.r13 * p.r13, a5 = p.c0 * (r2 * r2 * p.r13) * a.f5, a3 = p.c0 * c2 * (r2 * p.r13) * a.f3,
+               a2 = p.c0 * c3 * r2 * a.f2;
   p.m5 = -5.0 / 3.0 * a5 / mc;
   p.m3 = -a3 / mc;
   p.m2 = -2.0 / 3.0 * a2 / mc;
-  p.e3 = p.c0 * (r2 * p.r13) * (dc2 - 0.4 * c2 / eta);
+  p.e3 = p.c0 * (r2 * p.r13) * a.f3 * (dc2 - 0.4 * c2 / eta);
   p.e2 = -0.6 * a2 / eta;
 }
 
@@ -283,13 +306,15 @@ __device__ __forceinline__ void warp_sums(Sum (&v)[V], double* out) {
     }
   }
   constexpr int kCopies = 32 / V;  // lanes that hold the same value
-  if ((lane & (kCopies - 1)) == 0) out[first] = (double)v[0].h + ((double)v[0].m + (double)v[0].l);
+  // (an infinite term leaves NaN in the parts below the first)
+  if ((lane & (kCopies - 1)) == 0) out[first] = isfinite(v[0].h) ? (double)v[0].h + ((double)v[0].m + (double)v[0].l) : (double)v[0].h;
 }
 
 // `first` and `parts` lie in the shared memory of the cluster's first CTA: the constants, and the CTAs' partial sums.
+// The sums come divided by 2^top, top the largest exponent of the support.
 template <bool GRAD, bool PN3>
-__device__ void evaluate(const RefArgs& a, const cg::cluster_group& cluster, const Point* first, int64_t jhi, double* red,
-                         double* parts, Sums& out) {
+__device__ void evaluate(const RefArgs& a, const cg::cluster_group& cluster, const Point* first, int64_t jhi, int top,
+                         double* red, double* parts, Sums& out) {
   constexpr int V = GRAD ? 8 : 2;
   const int rank = (int)cluster.block_rank(), ranks = (int)cluster.num_blocks();
   const double m13 = first->m13, r13 = first->r13, c0 = first->c0, c2 = first->c2, c3 = first->c3, tc = first->tc,
@@ -297,7 +322,11 @@ __device__ void evaluate(const RefArgs& a, const cg::cluster_group& cluster, con
   Sum v[V] = {}, v2[2] = {};
 #pragma unroll 2
   for (int64_t j = a.jlo + rank * kThreads + threadIdx.x; j < jhi; j += ranks * kThreads) {
-    const float4 w = __ldg(a.w + j);
+    float4 w = __ldg(a.w + j);
+    {  // to the support's scale: 2^(e - top), nothing below 2^-126
+      const float unit = __int_as_float((max(__ldg(a.e + j) - top, -127) + 127) << 23);
+      w = make_float4(w.x * unit, w.y * unit, w.z * unit, w.w * unit);
+    }
     const double2 vt = __ldg(a.v + j);
     const double vv = m13 * vt.x, guess = r13 * vt.y;  // 1 / vv within two units in the last place
     const double iv = fma(guess, fma(-vv, guess, 1.0), guess);
@@ -384,17 +413,20 @@ __device__ void evaluate(const RefArgs& a, const cg::cluster_group& cluster, con
 }
 
 // Re(conj(zeta) dZ/dtheta_k) for zeta = (zr, zi), dZ/dtheta_k = i sum dPsi_k term (thread 0)
-__device__ __forceinline__ void derivatives(const RefArgs& a, const Point& p, const Sums& s, double zr, double zi, double (&d)[4]) {
+__device__ __forceinline__ void derivatives(const RefArgs& a, const Point& p, const Sums& s, int top, double zr, double zi,
+                                            double (&d)[4]) {
   double t[3][2];
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     t[0][c] = p.m5 * s.m5[c] + p.m3 * s.m3[c] + p.m2 * s.m2[c];
     t[1][c] = p.e3 * s.m3[c] + p.e2 * s.m2[c];
     t[2][c] = 2.0 * kPi * a.df * s.s1[c];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) t[k][c] = scalbn(t[k][c], top);
   }
 #pragma unroll
   for (int k = 0; k < 3; ++k) d[k] = zi * t[k][0] - zr * t[k][1];
-  d[3] = zr * s.z[1] - zi * s.z[0];  // dPsi/dphi_c = -1
+  d[3] = zr * scalbn(s.z[1], top) - zi * scalbn(s.z[0], top);  // dPsi/dphi_c = -1
 }
 
 __device__ __forceinline__ int64_t support_end(const RefArgs& a, double mc0, double eta0) {
@@ -410,6 +442,7 @@ template <int MODE, bool PN3>
 __global__ void __launch_bounds__(kThreads, 4) k_refine(RefArgs a) {
   // (of the cluster's first CTA: point, parts, s_jhi)
   __shared__ double red[(kThreads / 32) * 10], parts[kMaxRanks * 10];
+  __shared__ int red_e[kThreads / 32];
   __shared__ Point point;
   __shared__ int64_t s_jhi;
   const cg::cluster_group cluster = cg::this_cluster();
@@ -431,29 +464,33 @@ __global__ void __launch_bounds__(kThreads, 4) k_refine(RefArgs a) {
   if (lead && threadIdx.x == 32) make_point(a, th, point);
   cluster.sync();
   const int64_t jhi = min(*cluster.map_shared_rank(&s_jhi, 0), (int64_t)a.head->jmax);
-  // sigma^2 from the chunk sums and the last chunk's part
+  // the support's largest exponent, and sigma^2, from the chunks' and the last chunk's part
+  const int64_t whole = jhi / kThreads, part = whole * kThreads + threadIdx.x;
+  int top = kNoExponent;
+  for (int64_t k = a.jlo / kThreads + threadIdx.x; k < whole; k += kThreads) top = max(top, a.top[k]);
+  if (part < jhi && part >= a.jlo) top = max(top, a.e[part]);
+  top = block_max(top, red_e);
   double sig2 = 0.0;  // (the lead's thread 0)
   if (lead) {
-    const int64_t whole = jhi / kThreads, part = whole * kThreads + threadIdx.x;
     for (int64_t k = a.jlo / kThreads + threadIdx.x; k < whole; k += kThreads) sig2 += a.chunk[k];
     if (part < jhi && part >= a.jlo) sig2 += a.amp2[part];
     sig2 = block_sum(sig2, red);
   }
   Sums s;
   if (MODE == R_EVAL) {
-    evaluate<false, PN3>(a, cluster, first, jhi, red, sums, s);
+    evaluate<false, PN3>(a, cluster, first, jhi, top, red, sums, s);
     if (lead && threadIdx.x == 0) {
-      const double unit = scalbn(1.0, -amp_scale(a));
-      a.J[c] = (s.z[0] * s.z[0] + s.z[1] * s.z[1]) / sig2;
-      a.Z[2 * c] = s.z[0] * unit;
-      a.Z[2 * c + 1] = s.z[1] * unit;
+      const double zr = scalbn(s.z[0], top), zi = scalbn(s.z[1], top);
+      a.J[c] = (zr * zr + zi * zi) / sig2;
+      a.Z[2 * c] = zr;
+      a.Z[2 * c + 1] = zi;
     }
   } else if (MODE == R_ADJOINT) {
-    evaluate<true, PN3>(a, cluster, first, jhi, red, sums, s);
+    evaluate<true, PN3>(a, cluster, first, jhi, top, red, sums, s);
     if (lead && threadIdx.x == 0) {
-      const double unit = scalbn(1.0, amp_scale(a)), g = a.dJ[c];
+      const double g = a.dJ[c];
       double d[4];
-      derivatives(a, point, s, a.Z[2 * c] * unit, a.Z[2 * c + 1] * unit, d);
+      derivatives(a, point, s, top, a.Z[2 * c], a.Z[2 * c + 1], d);
 #pragma unroll
       for (int k = 0; k < 4; ++k) a.dtheta[4 * c + k] = g * 2.0 * d[k] / sig2;
     }
@@ -679,6 +716,8 @@ size_t carve(int64_t half, char* base, RefArgs* a) {
   a->amp2 = (double*)take(sizeof(double) * half);
   a->amp = a->amp2;
   a->chunk = (double*)take(sizeof(double) * ((half + kThreads - 1) / kThreads));
+  a->e = (int*)take(sizeof(int) * half);
+  a->top = (int*)take(sizeof(int) * ((half + kThreads - 1) / kThreads));
   return off;
 }
 
@@ -710,8 +749,14 @@ int prepare(const rb_refine_desc* d, const float* shat, const double* psd, const
   const double low = std::floor(d->f_low / a.df) - 1.0;
   a.jlo = low < 1.0 ? 1 : low < (double)half ? (int64_t)low : half;
   while (a.jlo < half && (double)a.jlo * a.df < d->f_low) ++a.jlo;
-  a.p53 = std::pow(kPi, -5.0 / 3.0);
-  a.p23 = std::pow(kPi, -2.0 / 3.0);
+  a.amp0 = 2.0 * std::pow(a.df, -2.0 / 3.0);  // 2 sqrt(df) df^(-7/6)
+  const double lo = (double)a.jlo, base = kPi * (lo * a.df);
+  a.r53 = std::pow(lo, 5.0 / 3.0);
+  a.r33 = lo;
+  a.r23 = std::pow(lo, 2.0 / 3.0);
+  a.f5 = std::pow(base, -5.0 / 3.0);
+  a.f3 = 1.0 / base;
+  a.f2 = std::pow(base, -2.0 / 3.0);
   a.pn = d->pn_order;
   a.n_cand = n_cand;
   a.steps = d->steps;
