@@ -46,6 +46,10 @@ constexpr double kFref = 100.0;
 constexpr double kEtaMin = 0.05;
 constexpr int kThreads = 128;
 constexpr int kMaxRanks = 8;  // CTAs (a cluster) that share a candidate's frequencies in value and adjoint, at most
+// Value and adjoint sum a candidate's frequencies in `strands` of every strands-th block of kThreads, as many as CTAs may
+// share a candidate at this n, each by one CTA from beginning to end, and the strands' sums in their order: a candidate's
+// result has the same bits however many CTAs its company leaves it. One CTA with all the strands loses 1 to 3 % to a single
+// sum (value and adjoint at n = 2^17, 456 candidates: 443 us before, 457 so; n = 2^19, 500: 1.70 and 1.72 ms).
 constexpr int kAscThreads = 256;  // threads of a candidate in the ascent
 // CTAs (a cluster) that these are spread over, in 20 steps of 512 candidates at n = 2^17 / of 64 at n = 2^15:
 // one 7.07 / 0.89 ms (two resident per SM, so that 512 leave the second wave two thirds empty), two 6.38 / 0.67,
@@ -76,6 +80,7 @@ struct RefArgs {
   double2* sh;
   double* amp;
   int64_t half, jlo;
+  int strands;  // 1, 2, 4 or 8
   double df;
   double amp0;                       // amp = amp0 j^(-7/6) / sqrt(S)
   double r53, r33, r23;              // jlo^(5/3), jlo, jlo^(2/3)
@@ -307,10 +312,12 @@ __device__ __forceinline__ void warp_sums(Sum (&v)[V], double* out) {
   }
   constexpr int kCopies = 32 / V;  // lanes that hold the same value
   // (an infinite term leaves NaN in the parts below the first)
-  if ((lane & (kCopies - 1)) == 0) out[first] = isfinite(v[0].h) ? (double)v[0].h + ((double)v[0].m + (double)v[0].l) : (double)v[0].h;
+  if ((lane & (kCopies - 1)) == 0)
+    out[first] = isfinite(v[0].h) ? (double)v[0].h + ((double)v[0].m + (double)v[0].l) : (double)v[0].h;
 }
 
-// `first` and `parts` lie in the shared memory of the cluster's first CTA: the constants, and the CTAs' partial sums.
+// `first` and `parts` lie in the shared memory of the cluster's first CTA: the constants, and the strands' sums. `red` holds
+// those of a CTA's warps in each of its strands.
 // The sums come divided by 2^top, top the largest exponent of the support.
 template <bool GRAD, bool PN3>
 __device__ void evaluate(const RefArgs& a, const cg::cluster_group& cluster, const Point* first, int64_t jhi, int top,
@@ -319,81 +326,87 @@ __device__ void evaluate(const RefArgs& a, const cg::cluster_group& cluster, con
   const int rank = (int)cluster.block_rank(), ranks = (int)cluster.num_blocks();
   const double m13 = first->m13, r13 = first->r13, c0 = first->c0, c2 = first->c2, c3 = first->c3, tc = first->tc,
                phic = first->phic;
-  Sum v[V] = {}, v2[2] = {};
+  constexpr int NV = GRAD && PN3 ? V + 2 : V;
+  const int own = a.strands / ranks;
+  __syncthreads();  // (red may still be read)
+#pragma unroll 1
+  for (int q = 0; q < own; ++q) {
+    Sum v[V] = {}, v2[2] = {};
 #pragma unroll 2
-  for (int64_t j = a.jlo + rank * kThreads + threadIdx.x; j < jhi; j += ranks * kThreads) {
-    float4 w = __ldg(a.w + j);
-    {  // to the support's scale: 2^(e - top), nothing below 2^-126
-      const float unit = __int_as_float((max(__ldg(a.e + j) - top, -127) + 127) << 23);
-      w = make_float4(w.x * unit, w.y * unit, w.z * unit, w.w * unit);
-    }
-    const double2 vt = __ldg(a.v + j);
-    const double vv = m13 * vt.x, guess = r13 * vt.y;  // 1 / vv within two units in the last place
-    const double iv = fma(guess, fma(-vv, guess, 1.0), guess);
-    const double iv2 = iv * iv, iv3 = iv2 * iv, iv5 = iv3 * iv2;
-    double phase = __ldg(a.x + j) * tc - phic - 0.25 * kPi;
-    if constexpr (GRAD) {  // (rounded as in the ascent)
-      const double in = __fma_rn(c2, iv3, iv5);
-      phase = __dadd_rn(phase, __dmul_rn(c0, PN3 ? __fma_rn(c3, iv2, in) : in));
-    } else {
-      phase += PN3 ? c0 * (iv5 + c2 * iv3 + c3 * iv2) : c0 * (iv5 + c2 * iv3);
-    }
-    // the nearest whole number of turns, by an addition that leaves no fraction bits (|turns| < 2^51)
-    const double k = fma(phase, 1.0 / (2.0 * kPi), 6755399441055744.0) - 6755399441055744.0;
-    phase -= 2.0 * kPi * k;
-    const float psi = (float)phase;
-    float sn, cs;
-    sincosf(psi, &sn, &cs);
-    // term = w exp(i Psi)
-    Pair t[2];
-    float e;
-    {
-      const float p = __fmul_rn(w.x, cs), q = __fmul_rn(w.y, sn);
-      t[0].h = two_sum(p, -q, e);
-      t[0].l = __fadd_rn(e, __fsub_rn(__fmaf_rn(w.z, cs, __fmaf_rn(w.x, cs, -p)), __fmaf_rn(w.w, sn, __fmaf_rn(w.y, sn, -q))));
-    }
-    {
-      const float p = __fmul_rn(w.x, sn), q = __fmul_rn(w.y, cs);
-      t[1].h = two_sum(p, q, e);
-      t[1].l = __fadd_rn(e, __fadd_rn(__fmaf_rn(w.z, sn, __fmaf_rn(w.x, sn, -p)), __fmaf_rn(w.w, cs, __fmaf_rn(w.y, cs, -q))));
-    }
-    float4 g;
-    float2 g2;
-    if constexpr (GRAD) g = __ldg(a.g + j);
-    if constexpr (GRAD && PN3) g2 = __ldg(a.g2 + j);
+    for (int j = (int)a.jlo + (rank * own + q) * kThreads + (int)threadIdx.x; j < (int)jhi; j += a.strands * kThreads) {  // (< 2^20)
+      float4 w = __ldg(a.w + j);
+      {  // to the support's scale: 2^(e - top), nothing below 2^-126
+        const float unit = __int_as_float((max(__ldg(a.e + j) - top, -127) + 127) << 23);
+        w = make_float4(w.x * unit, w.y * unit, w.z * unit, w.w * unit);
+      }
+      const double2 vt = __ldg(a.v + j);
+      const double vv = m13 * vt.x, guess = r13 * vt.y;  // 1 / vv within two units in the last place
+      const double iv = fma(guess, fma(-vv, guess, 1.0), guess);
+      const double iv2 = iv * iv, iv3 = iv2 * iv, iv5 = iv3 * iv2;
+      double phase = __ldg(a.x + j) * tc - phic - 0.25 * kPi;
+      if constexpr (GRAD) {  // (rounded as in the ascent)
+        const double in = __fma_rn(c2, iv3, iv5);
+        phase = __dadd_rn(phase, __dmul_rn(c0, PN3 ? __fma_rn(c3, iv2, in) : in));
+      } else {
+        phase += PN3 ? c0 * (iv5 + c2 * iv3 + c3 * iv2) : c0 * (iv5 + c2 * iv3);
+      }
+      // the nearest whole number of turns, by an addition that leaves no fraction bits (|turns| < 2^51)
+      const double k = fma(phase, 1.0 / (2.0 * kPi), 6755399441055744.0) - 6755399441055744.0;
+      phase -= 2.0 * kPi * k;
+      const float psi = (float)phase;
+      float sn, cs;
+      sincosf(psi, &sn, &cs);
+      // term = w exp(i Psi)
+      Pair t[2];
+      float e;
+      {
+        const float p = __fmul_rn(w.x, cs), q = __fmul_rn(w.y, sn);
+        t[0].h = two_sum(p, -q, e);
+        t[0].l = __fadd_rn(e, __fsub_rn(__fmaf_rn(w.z, cs, __fmaf_rn(w.x, cs, -p)), __fmaf_rn(w.w, sn, __fmaf_rn(w.y, sn, -q))));
+      }
+      {
+        const float p = __fmul_rn(w.x, sn), q = __fmul_rn(w.y, cs);
+        t[1].h = two_sum(p, q, e);
+        t[1].l = __fadd_rn(e, __fadd_rn(__fmaf_rn(w.z, sn, __fmaf_rn(w.x, sn, -p)), __fmaf_rn(w.w, cs, __fmaf_rn(w.y, cs, -q))));
+      }
+      float4 g;
+      float2 g2;
+      if constexpr (GRAD) g = __ldg(a.g + j);
+      if constexpr (GRAD && PN3) g2 = __ldg(a.g2 + j);
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      add(v[c], t[c].h, t[c].l);
-      if constexpr (GRAD) {
-        const float fj = (float)(int)j;  // exact
-        const float p = __fmul_rn(t[c].h, fj);
-        add(v[2 + c], p, __fmaf_rn(t[c].l, fj, __fmaf_rn(t[c].h, fj, -p)));
-        const Pair x5 = mul(t[c], g.x, g.y), x3 = mul(t[c], g.z, g.w);
-        add(v[4 + c], x5.h, x5.l);
-        add(v[6 + c], x3.h, x3.l);
-        if constexpr (PN3) {
-          const Pair x2 = mul(t[c], g2.x, g2.y);
-          add(v2[c], x2.h, x2.l);
+      for (int c = 0; c < 2; ++c) {
+        add(v[c], t[c].h, t[c].l);
+        if constexpr (GRAD) {
+          const float fj = (float)j;  // exact
+          const float p = __fmul_rn(t[c].h, fj);
+          add(v[2 + c], p, __fmaf_rn(t[c].l, fj, __fmaf_rn(t[c].h, fj, -p)));
+          const Pair x5 = mul(t[c], g.x, g.y), x3 = mul(t[c], g.z, g.w);
+          add(v[4 + c], x5.h, x5.l);
+          add(v[6 + c], x3.h, x3.l);
+          if constexpr (PN3) {
+            const Pair x2 = mul(t[c], g2.x, g2.y);
+            add(v2[c], x2.h, x2.l);
+          }
         }
       }
     }
+    // sums over a warp in parts, over the warps and the strands in FP64
+    double* const sums = red + (q * (kThreads / 32) + (threadIdx.x >> 5)) * NV;
+    warp_sums<V>(v, sums);
+    if constexpr (GRAD && PN3) warp_sums<2>(v2, sums + V);
   }
-  // sums over a warp in parts, over the warps and the cluster's CTAs in FP64
-  constexpr int NV = GRAD && PN3 ? V + 2 : V;
-  __syncthreads();  // (red may still be read from the pass before)
-  warp_sums<V>(v, red + (threadIdx.x >> 5) * NV);
-  if constexpr (GRAD && PN3) warp_sums<2>(v2, red + (threadIdx.x >> 5) * NV + V);
   __syncthreads();
-  if (threadIdx.x < NV) {
-    double t = red[threadIdx.x];
-    for (int k = 1; k < kThreads / 32; ++k) t += red[k * NV + threadIdx.x];
-    parts[rank * 10 + threadIdx.x] = t;
+  if (threadIdx.x < own * NV) {
+    const int q = threadIdx.x / NV, i = threadIdx.x % NV;
+    double t = red[q * (kThreads / 32) * NV + i];
+    for (int w = 1; w < kThreads / 32; ++w) t += red[(q * (kThreads / 32) + w) * NV + i];
+    parts[(rank * own + q) * 10 + i] = t;
   }
   cluster.sync();
   if (rank != 0) return;
   if (threadIdx.x < NV) {
     double t = parts[threadIdx.x];
-    for (int k = 1; k < ranks; ++k) t += parts[k * 10 + threadIdx.x];
+    for (int q = 1; q < a.strands; ++q) t += parts[q * 10 + threadIdx.x];
     red[threadIdx.x] = t;
   }
   __syncthreads();
@@ -439,9 +452,9 @@ __device__ __forceinline__ int64_t support_end(const RefArgs& a, double mc0, dou
 }
 
 template <int MODE, bool PN3>
-__global__ void __launch_bounds__(kThreads, 4) k_refine(RefArgs a) {
+__global__ void __launch_bounds__(kThreads, MODE == R_EVAL ? 8 : 5) k_refine(RefArgs a) {
   // (of the cluster's first CTA: point, parts, s_jhi)
-  __shared__ double red[(kThreads / 32) * 10], parts[kMaxRanks * 10];
+  __shared__ double red[kMaxRanks * (kThreads / 32) * 10], parts[kMaxRanks * 10];
   __shared__ int red_e[kThreads / 32];
   __shared__ Point point;
   __shared__ int64_t s_jhi;
@@ -749,6 +762,8 @@ int prepare(const rb_refine_desc* d, const float* shat, const double* psd, const
   const double low = std::floor(d->f_low / a.df) - 1.0;
   a.jlo = low < 1.0 ? 1 : low < (double)half ? (int64_t)low : half;
   while (a.jlo < half && (double)a.jlo * a.df < d->f_low) ++a.jlo;
+  a.strands = 1;
+  while (a.strands < kMaxRanks && half / (2 * a.strands * kThreads) >= 32) a.strands *= 2;
   a.amp0 = 2.0 * std::pow(a.df, -2.0 / 3.0);  // 2 sqrt(df) df^(-7/6)
   const double lo = (double)a.jlo, base = kPi * (lo * a.df);
   a.r53 = std::pow(lo, 5.0 / 3.0);
@@ -799,7 +814,7 @@ int run(const RefArgs& a, cudaStream_t st) {
     // 456: 1318 / 1550 / 1508 / 1515; n = 2^17, 64: 303 / 224 / 207 / 220, 227: 358 / 301 / 391 / 386; n = 2^14, 64:
     // 157 / 150 / 150 / 174, 300: 168 / 184 / 230 / 284.
     int ranks = 1;
-    while (ranks < kMaxRanks && 2 * ranks * a.n_cand <= 512 && a.half / (2 * ranks * kThreads) >= 32) ranks *= 2;
+    while (ranks < a.strands && 2 * ranks * a.n_cand <= 512) ranks *= 2;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)ranks;
