@@ -421,10 +421,12 @@ int rb_tune_stage1(const rb_filter_desc* desc, const rb_basis* basis, const floa
 
 /*
  * rb_tune_fft - autotuner of the FFT schedule of the basis filter (rb_basis_filter, and inside
- * rb_filter / rb_filter_batch / rb_filter_plain): times every variant of RB_FFT_VARIANTS (columns
- * per CTA of the two four-step passes of short transforms, and the megabytes of the intermediate that
- * are to stay in L2) on this desc's basis and s_hat, and remembers the fastest for (n, w) in a process-wide
- * table (variant 0 when untuned). Measurement support, not in the paper.
+ * rb_filter / rb_filter_batch / rb_filter_plain). Few rows take two four-step passes, which have
+ * RB_FFT_VARIANTS schedules (columns per CTA of the two passes, and the megabytes of the intermediate
+ * that are to stay in L2): every one is timed on this desc's basis and s_hat, and the fastest is
+ * remembered for the passes of (n, w) in a process-wide table (variant 0 when untuned). Many rows (2^22
+ * points in all from n = 2^17 on, 2^23 from n = 2^14 on) take one fused launch, which has one schedule:
+ * its time fills times_ms, *chosen is 0 and nothing is remembered. Measurement support, not in the paper.
  *   s_hat: [n/2] complex device (rb_whiten output). times_ms: HOST [RB_FFT_VARIANTS] mean ms of one
  *   basis filter. chosen: HOST, the selected variant. Synchronises `stream`.
  *   Errors: RB_ERR_BAD_INPUT (NULL argument, basis not matching desc), RB_ERR_OOM (workspace).
@@ -432,7 +434,7 @@ int rb_tune_stage1(const rb_filter_desc* desc, const rb_basis* basis, const floa
 #define RB_FFT_VARIANTS 8
 int rb_tune_fft(const rb_filter_desc* desc, const rb_basis* basis, const float* s_hat, double* times_ms,
                 int32_t* chosen, void* workspace, size_t workspace_bytes, void* stream);
-/* rb_set_fft_variant - pin the FFT schedule variant used for desc's (n, w). Host only. */
+/* rb_set_fft_variant - pin the variant of the two passes for desc's (n, w). Host only. */
 int rb_set_fft_variant(const rb_filter_desc* desc, int32_t variant);
 
 /* Stages of rb_filter timed by the profiler (CUDA events recorded on the call's stream). */

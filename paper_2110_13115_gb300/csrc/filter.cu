@@ -19,12 +19,12 @@
 using namespace rbfft;
 
 namespace rbseries {  // series_*.cu
-int launch_bank_short(int log2n, const Args& a, int rows_l2, int rows_ws, cudaStream_t st);
-int launch_bank_long(int log2n, const Args& a, int rows_l2, int rows_ws, cudaStream_t st);
-int launch_plain_short(int log2n, const Args& a, int rows_l2, int rows_ws, cudaStream_t st);
-int launch_plain_long(int log2n, const Args& a, int rows_l2, int rows_ws, cudaStream_t st);
-int launch_fold_short(int log2n, const Args& a, int rows_l2, int rows_ws, cudaStream_t st);
-int launch_fold_long(int log2n, const Args& a, int rows_l2, int rows_ws, cudaStream_t st);
+int launch_bank_short(int log2n, const Args& a, int rows_ws, cudaStream_t st);
+int launch_bank_long(int log2n, const Args& a, int rows_ws, cudaStream_t st);
+int launch_plain_short(int log2n, const Args& a, int rows_ws, cudaStream_t st);
+int launch_plain_long(int log2n, const Args& a, int rows_ws, cudaStream_t st);
+int launch_fold_short(int log2n, const Args& a, int rows_ws, cudaStream_t st);
+int launch_fold_long(int log2n, const Args& a, int rows_ws, cudaStream_t st);
 }  // namespace rbseries
 
 namespace {
@@ -650,8 +650,7 @@ bool use_fused(const rb::Geometry& g, int64_t nvec) {
   return g.n >= (1 << 14) && g.n * nvec >= (int64_t)(g.n >= (1 << 17) ? 1 << 22 : 1 << 23) && rb::fft_fused_enabled();
 }
 
-int series_run(const rb::Geometry& g, const rb::Workspace& ws, rbseries::Args a, int kind, int mb,
-               cudaStream_t st) {
+int series_run(const rb::Geometry& g, const rb::Workspace& ws, rbseries::Args a, int kind, cudaStream_t st) {
   a.X = ws.X;
   a.w2a = ws.tables.w2a;
   a.w4 = ws.tables.w4;
@@ -660,16 +659,16 @@ int series_run(const rb::Geometry& g, const rb::Workspace& ws, rbseries::Args a,
   a.log2w = rb_ilog2(a.w);
   a.align_rows = (((uintptr_t)a.rows | (uintptr_t)a.shat) & 15) == 0;
   a.align_beta = ((uintptr_t)a.beta & 15) == 0;
-  const int log2n = rb_ilog2(g.n), rows_l2 = (int)std::max<int64_t>(1, ((int64_t)mb << 20) / (g.n * 8));
-  using Launch = int (*)(int, const rbseries::Args&, int, int, cudaStream_t);
+  const int log2n = rb_ilog2(g.n);
+  using Launch = int (*)(int, const rbseries::Args&, int, cudaStream_t);
   constexpr Launch launch[3][2] = {{rbseries::launch_bank_short, rbseries::launch_bank_long},
                                    {rbseries::launch_plain_short, rbseries::launch_plain_long},
                                    {rbseries::launch_fold_short, rbseries::launch_fold_long}};
-  return launch[kind][log2n > 16](log2n, a, rows_l2, ws.vc, st);
+  return launch[kind][log2n > 16](log2n, a, ws.vc, st);
 }
 
-// FFT schedule variants of the basis filter: columns per CTA of pass A and pass B, and the size
-// in MB of a four-step chunk's intermediate X (which stays in L2 between the passes).
+// Schedule variants of the two radix-16 passes: columns per CTA of pass A and pass B, and the size in MB of a
+// four-step chunk's intermediate X (which stays in L2 between the passes). The fused launch has one schedule.
 struct FftVariant {
   int ga, gb, mb;
 };
@@ -682,7 +681,7 @@ int chunk_vectors(const rb::Geometry& g, const rb::Workspace& ws, const FftVaria
 }
 
 std::mutex g_fft_mu;
-std::map<std::pair<int64_t, int>, int> g_fft_choice;  // (n, w) -> variant
+std::map<std::pair<int64_t, int>, int> g_fft_choice;  // (n, w) -> variant of the radix-16 passes
 
 int fft_variant_for(int64_t n, int w) {
   std::lock_guard<std::mutex> lk(g_fft_mu);
@@ -732,7 +731,7 @@ static int bank_filter_v(const Geometry& g, const Workspace& ws, const float2* r
     a.w = w;
     a.beta = beta;
     a.beta_avg = bavg;
-    return series_run(g, ws, a, rbseries::KIND_BANK, v.mb, st);
+    return series_run(g, ws, a, rbseries::KIND_BANK, st);
   }
   const int vc = chunk_vectors(g, ws, v);
   for (int64_t v0 = 0; v0 < nvec; v0 += vc) {
@@ -776,8 +775,11 @@ int tune_fft(const Geometry& g, const Workspace& ws, const float2* rows, int64_t
   cudaEvent_t e0, e1;
   RB_CUDA_TRY(cudaEventCreate(&e0));
   RB_CUDA_TRY(cudaEventCreate(&e1));
+  // rows that take the fused launch have nothing to choose: one time serves for all, and the choice of the radix-16
+  // passes, which fewer rows of this n and w take, stays what it was
+  const bool one = use_fused(g, nvec);
   int rc = RB_OK, best = 0;
-  for (int v = 0; v < RB_FFT_VARIANTS && rc == RB_OK; ++v) {
+  for (int v = 0; v < (one ? 1 : RB_FFT_VARIANTS) && rc == RB_OK; ++v) {
     const int reps = 3;
     rc = bank_filter_v(g, ws, rows, nvec, shat, beta, bavg, w, kFftVariants[v], st);  // warm-up
     if (rc == RB_OK && cudaEventRecord(e0, st) != cudaSuccess) rc = RB_ERR_CUDA;
@@ -799,6 +801,10 @@ int tune_fft(const Geometry& g, const Workspace& ws, const float2* rows, int64_t
     return rc;
   }
   *chosen = best;
+  if (one) {
+    for (int v = 1; v < RB_FFT_VARIANTS; ++v) ms[v] = ms[0];
+    return RB_OK;
+  }
   return set_fft_variant(g, w, best);
 }
 
@@ -818,7 +824,7 @@ int plain_filter(const Geometry& g, const Workspace& ws, const float2* tmpl, int
     a.thr2 = thr2;
     a.sample_offset = sample_offset;
     a.block_id = block_id;
-    return series_run(g, ws, a, rbseries::KIND_PLAIN, v.mb, st);
+    return series_run(g, ws, a, rbseries::KIND_PLAIN, st);
   }
   const int vc = chunk_vectors(g, ws, v);
   for (int64_t v0 = 0; v0 < T; v0 += vc) {
@@ -880,7 +886,7 @@ int folded_stage1(const Geometry& gm, const Workspace& wm, const float2* tmpl, i
       a.cap = cap;
       a.thr2 = thr2;
       a.block_id = block_id;
-      const int rc = series_run(gm, wm, a, rbseries::KIND_FOLD, 32, st);
+      const int rc = series_run(gm, wm, a, rbseries::KIND_FOLD, st);
       if (rc) return rc;
     }
     return RB_OK;

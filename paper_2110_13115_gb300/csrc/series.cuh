@@ -612,10 +612,9 @@ inline int sm_count() {
   return sms;
 }
 
-// rows_l2: rows of X that may stay in L2 (the ring is about that long, and long enough for the order);
-// rows_ws: rows that the workspace holds.
+// rows_ws: rows of X that the workspace holds. The ring is as long as the order needs, so that X stays in L2.
 template <int LOG2N, int WARPS, int KIND>
-int launch(Args a, int rows_l2, int rows_ws, cudaStream_t st) {
+int launch(Args a, int rows_ws, cudaStream_t st) {
   using S = Shape<LOG2N, WARPS>;
   auto kern = k_series<LOG2N, WARPS, KIND>;
   RB_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmem));
@@ -625,7 +624,7 @@ int launch(Args a, int rows_l2, int rows_ws, cudaStream_t st) {
   // first item; the ring holds the rows between the first A item and the last B item in flight.
   const auto rows_of = [&](int64_t t) { return (int)((t + S::ITEMS - 1) / S::ITEMS); };
   a.lag = (int)std::min<int64_t>(items, S::ITEMS + 1 + grid);
-  const int want = std::max(rows_l2, rows_of(a.lag) + 2 + rows_of(grid / 2));
+  const int want = rows_of(a.lag) + 2 + rows_of(grid / 2);
   // a power of two: of at least nvec rows (no slot is used twice), or of what the workspace holds
   a.log2ring = 0;
   while ((1 << a.log2ring) < a.nvec && (2 << a.log2ring) <= (a.nvec <= rows_ws ? 2 * a.nvec : rows_ws) && (1 << a.log2ring) < want) ++a.log2ring;

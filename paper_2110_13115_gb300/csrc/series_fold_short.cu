@@ -3,11 +3,11 @@
 
 namespace rbseries {
 
-int launch_fold_short(int log2n, const Args& a, int rows_l2, int rows_ws, cudaStream_t st) {
+int launch_fold_short(int log2n, const Args& a, int rows_ws, cudaStream_t st) {
   switch (log2n) {
-    case 14: return launch<14, 4, KIND_FOLD>(a, rows_l2, rows_ws, st);
-    case 15: return launch<15, 4, KIND_FOLD>(a, rows_l2, rows_ws, st);
-    case 16: return launch<16, 4, KIND_FOLD>(a, rows_l2, rows_ws, st);
+    case 14: return launch<14, 4, KIND_FOLD>(a, rows_ws, st);
+    case 15: return launch<15, 4, KIND_FOLD>(a, rows_ws, st);
+    case 16: return launch<16, 4, KIND_FOLD>(a, rows_ws, st);
   }
   rb::set_detail("fused transform of 2^%d points", log2n);
   return RB_ERR_UNSUPPORTED;
