@@ -161,8 +161,8 @@ int rb_whiten(const rb_filter_desc* desc, const float* strain, const double* psd
  *   beta_avg: [k][n/(2w)] complex output (index i - n/(2w)).
  *   Errors: RB_ERR_BAD_INPUT (desc invalid, basis not matching desc, NULL s_hat or beta_avg),
  *   RB_ERR_OOM (workspace smaller than rb_filter_plan's size or not 256-byte aligned).
- *   Enqueue only: a bounded device-side wait that gave up (RB_ERR_TIMEOUT of the calls that read the
- *   status) leaves beta incomplete without a report here.
+ *   Enqueue only: where a bounded device-side wait gave up (RB_ERR_TIMEOUT of the calls that read the
+ *   status), every value of beta and beta_avg is NaN.
  */
 int rb_basis_filter(const rb_filter_desc* desc, const rb_basis* basis, const float* s_hat,
                     float* beta, float* beta_avg, void* workspace, size_t workspace_bytes,
@@ -429,7 +429,8 @@ int rb_tune_stage1(const rb_filter_desc* desc, const rb_basis* basis, const floa
  * its time fills times_ms, *chosen is 0 and nothing is remembered. Measurement support, not in the paper.
  *   s_hat: [n/2] complex device (rb_whiten output). times_ms: HOST [RB_FFT_VARIANTS] mean ms of one
  *   basis filter. chosen: HOST, the selected variant. Synchronises `stream`.
- *   Errors: RB_ERR_BAD_INPUT (NULL argument, basis not matching desc), RB_ERR_OOM (workspace).
+ *   Errors: RB_ERR_BAD_INPUT (NULL argument, basis not matching desc), RB_ERR_OOM (workspace),
+ *   RB_ERR_TIMEOUT (a bounded device-side wait ran out).
  */
 #define RB_FFT_VARIANTS 8
 int rb_tune_fft(const rb_filter_desc* desc, const rb_basis* basis, const float* s_hat, double* times_ms,

@@ -677,6 +677,12 @@ int rb_tune_fft(const rb_filter_desc* desc, const rb_basis* basis, const float* 
   if ((rc = tune_fft(g, ws, (const float2*)basis->vectors, desc->k, (const float2*)s_hat, ws.beta, ws.bavg,
                      desc->w, times_ms, &best, st)))
     return rc;
+  Status s;
+  if ((rc = read_status(ws, &s, st))) return rc;
+  if (s.flags & RB_FLAG_TIMEOUT) {
+    set_detail("a bounded device-side wait of the transforms timed out");
+    return RB_ERR_TIMEOUT;
+  }
   *chosen = best;
   return RB_OK;
 }

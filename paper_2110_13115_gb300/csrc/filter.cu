@@ -650,6 +650,8 @@ bool use_fused(const rb::Geometry& g, int64_t nvec) {
   return g.n >= (1 << 14) && g.n * nvec >= (int64_t)(g.n >= (1 << 17) ? 1 << 22 : 1 << 23) && rb::fft_fused_enabled();
 }
 
+std::atomic<int> g_withhold{0};  // fused launches left whose part B waits in vain (failure-detection test)
+
 int series_run(const rb::Geometry& g, const rb::Workspace& ws, rbseries::Args a, int kind, cudaStream_t st) {
   a.X = ws.X;
   a.w2a = ws.tables.w2a;
@@ -659,6 +661,10 @@ int series_run(const rb::Geometry& g, const rb::Workspace& ws, rbseries::Args a,
   a.log2w = rb_ilog2(a.w);
   a.align_rows = (((uintptr_t)a.rows | (uintptr_t)a.shat) & 15) == 0;
   a.align_beta = ((uintptr_t)a.beta & 15) == 0;
+  int left = g_withhold.load();
+  while (left > 0 && !g_withhold.compare_exchange_weak(left, left - 1)) {
+  }
+  a.withhold = left > 0 ? 1u : 0u;
   const int log2n = rb_ilog2(g.n);
   using Launch = int (*)(int, const rbseries::Args&, int, cudaStream_t);
   constexpr Launch launch[3][2] = {{rbseries::launch_bank_short, rbseries::launch_bank_long},
@@ -973,5 +979,13 @@ int pack_coeff(const rb_filter_desc& d, const rb_basis& b, const Geometry& g, vo
 // between the two and for timing.
 extern "C" int rbx_set_fft_radix32(int mode) {
   rb::g_fused.store(mode > 0);
+  return 0;
+}
+
+// Host-only test hook (not part of the C ABI): in the next n fused launches part B waits for a count that part A does not
+// reach, so the bounded wait runs out, the launch stops and the context stays usable. Used by the failure-detection
+// test; no other code calls it.
+extern "C" int rbx_series_withhold(int n) {
+  g_withhold.store(n > 0 ? n : 0);
   return 0;
 }

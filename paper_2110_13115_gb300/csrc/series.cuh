@@ -27,7 +27,8 @@
 // Order and dependencies. Tickets are taken in increasing order by CTAs that are running, a CTA never
 // waits while it holds results that it has not announced, and an item depends on items of lower tickets
 // only: the lowest unfinished ticket can always finish, whatever else runs on the GPU. Waits are bounded
-// all the same (RB_FLAG_TIMEOUT).
+// all the same (RB_FLAG_TIMEOUT); a basis filter whose launch gave up fills beta and the bin means with NaN, as not
+// every caller of it reads the flag.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -74,6 +75,7 @@ struct Args {
   int block_id;
   int align_rows;  // rows and shat lie on 16-byte boundaries (else on 8-byte ones)
   int align_beta;
+  unsigned withhold;  // failure-detection test: part B waits for one count more than there is (rbx_series_withhold)
 };
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
@@ -250,7 +252,7 @@ __global__ void __launch_bounds__(32 * WARPS, WARPS == 4 ? 3 : 1) k_series(const
     unsigned item;
     const int part = part_of(t, items, (unsigned)a.lag, &item);
     const unsigned vec = item / I, gen = vec >> a.log2ring;
-    return {(part ? done_a : done_b) + (vec & slot_mask), part ? (gen + 1) * (unsigned)(I * WARPS) : gen * (unsigned)I};
+    return {(part ? done_a : done_b) + (vec & slot_mask), part ? (gen + 1) * (unsigned)(I * WARPS) + a.withhold : gen * (unsigned)I};
   };
   // (one thread) until the ticket may start; false when it never will
   auto wait_ready = [&](unsigned t) {
@@ -592,10 +594,24 @@ __global__ void __launch_bounds__(32 * WARPS, WARPS == 4 ? 3 : 1) k_series(const
   if (threadIdx.x == 0) {
     // the last CTA leaves the words zero for the next launch (an aborted launch: the next call's set-up does)
     fence_gpu();
-    if (atomicAdd(a.sync + 1, 1u) == gridDim.x - 1 && !ld_acquire(a.sync + 2)) {
+    const bool last = atomicAdd(a.sync + 1, 1u) == gridDim.x - 1;
+    fence_gpu();
+    const bool gave_up = last && ld_acquire(a.sync + 2);
+    if (last && !gave_up) {
       for (int i = 0; i < 2 << a.log2ring; ++i) done_a[i] = 0;
       a.sync[0] = 0;
       a.sync[1] = 0;
+    }
+    s_abort = gave_up;
+  }
+  if constexpr (KIND == KIND_BANK) {  // (the other kinds' callers read the flag)
+    __syncthreads();
+    if (s_abort) {
+      const float nan = __int_as_float(0x7fffffff);
+      const int64_t rows = a.nvec, bins = HALF >> a.log2w;
+      for (int64_t i = threadIdx.x; i < rows * bins; i += NT) a.beta_avg[a.vec0 * bins + i] = make_float2(nan, nan);
+      if (a.beta)
+        for (int64_t i = threadIdx.x; i < rows * HALF; i += NT) a.beta[a.vec0 * HALF + i] = make_float2(nan, nan);
     }
   }
 }
