@@ -14,7 +14,7 @@
 // barrier and its results leave as runs of L / 4 contiguous bytes; in part B the lanes span the columns,
 // which makes the loads, the stores of beta and the bin sums contiguous.
 //
-// What bounds it, and what was measured (n = 2^19, 201 rows, w = 8): 538 us against 892 us for two radix-32 launches
+// What bounds it, and what was measured (n = 2^19, 201 rows, w = 8): 520 us against 892 us for two radix-32 launches
 // per chunk of 8 rows, which it replaces (132 us are the rows' HBM bytes). The launches lost 512 work items to
 // 456 resident CTAs, a gap and a ramp each. Three CTAs of 128 threads fit an SM (168 registers, 74 KB); the issue
 // slots are busy 30 % of the time and the long straight-line code of an item (about 2000 instructions a warp) is what
@@ -22,7 +22,8 @@
 // step, so that they fetch it together, brought the fetch stalls from 2.9 to 0.4 cycles per instruction and as much
 // waiting for each other's shared-memory and FP32 phases (3.27 us); two CTAs with 255 registers and a separate
 // exchange buffer: 3.2 us; L2 residency hints on X: no change; fewer instructions (no spare cases): 2.75 us, and with
-// short copy loops and exchange addresses 2.69 us.
+// short copy loops and exchange addresses 2.69 us, without the twiddles' row of ones in shared memory 2.58 us (and at 2^20,
+// where that row left room for two CTAs an SM only, 6.63 -> 6.00 us a row).
 //
 // Order and dependencies. Tickets are taken in increasing order by CTAs that are running, a CTA never
 // waits while it holds results that it has not announced, and an item depends on items of lower tickets
@@ -117,8 +118,11 @@ struct Shape {
   // the tile, then the exchange in its place: 16 bytes (two columns) per point, the points of a run of 32
   // permuted by the run's number, which spreads a quarter warp's stores and loads over all banks in both parts
   static constexpr int kTile = TP * 8;
-  static constexpr int kTw = N2 * 8, kRoots = (N1 / 4 + 128) * 8;
+  // stage-2 twiddles of the powers 1 .. SA - 1 (at 2^20 points the row of ones would cost the third CTA of an SM)
+  static constexpr int kTw = (SA - 1) * 32 * 8, kRoots = (N1 / 4 + 128) * 8;
   static constexpr int kSmem = kTile + kTw + kRoots;
+  static constexpr int kCtas = WARPS == 4 ? 3 : 1;  // per SM: 228 KB, of which a CTA takes 1 KB and its static variables more
+  static_assert(kCtas * (kSmem + 1024 + 256) <= 228 * 1024, "resident CTAs");
   // chunk swizzle of part A's tile (16-byte units, U per row): the eight lanes of a 16-byte load, which
   // read eight consecutive rows of one pair (four rows of two pairs when SA = 4), hit distinct banks
   static constexpr int U = CA / 2;
@@ -215,14 +219,14 @@ static __device__ __noinline__ void plain_window(const Args& a, float2 re, float
 }
 
 template <int LOG2N, int WARPS, int KIND>
-__global__ void __launch_bounds__(32 * WARPS, WARPS == 4 ? 3 : 1) k_series(const __grid_constant__ Args a) {
+__global__ void __launch_bounds__(32 * WARPS, Shape<LOG2N, WARPS>::kCtas) k_series(const __grid_constant__ Args a) {
   using S = Shape<LOG2N, WARPS>;
   constexpr bool FULL = KIND == KIND_FOLD;
   constexpr int N1 = S::N1, N2 = S::N2, NT = S::NT, TP = S::TP, I = S::ITEMS, SA = S::SA, SB = S::SB;
   constexpr int64_t N = (int64_t)1 << LOG2N, HALF = N / 2;
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned char* const tile = smem;
-  float2* const tw = reinterpret_cast<float2*>(smem + S::kTile);  // [r][32]: exp(2 pi i j r / n2)
+  float2* const tw = reinterpret_cast<float2*>(smem + S::kTile);  // [r - 1][32]: exp(2 pi i j r / n2)
   float2* const roots = reinterpret_cast<float2*>(smem + S::kTile + S::kTw);
   __shared__ unsigned s_next[2];
   __shared__ int s_ready[2], s_abort;
@@ -325,7 +329,7 @@ __global__ void __launch_bounds__(32 * WARPS, WARPS == 4 ? 3 : 1) k_series(const
     }
   };
   if (threadIdx.x == 0) s_next[0] = atomicAdd(a.sync, 1u);
-  for (int e = threadIdx.x; e < N2; e += NT) tw[e] = a.w2a[(e & 31) * (SA + 1) + (e >> 5)];
+  for (int e = threadIdx.x; e < N2 - 32; e += NT) tw[e] = a.w2a[(e & 31) * (SA + 1) + (e >> 5) + 1];
   for (int e = threadIdx.x; e < N1 / 4 + 128; e += NT) roots[e] = a.w4[e];
   if (threadIdx.x == 0) s_abort = s_next[0] < total && !wait_ready(s_next[0]);
   __syncthreads();
@@ -438,7 +442,7 @@ __global__ void __launch_bounds__(32 * WARPS, WARPS == 4 ? 3 : 1) k_series(const
 #pragma unroll
       for (int b = 0; b < 32 / SA; ++b) {
 #pragma unroll
-        for (int r = 1; r < SA; ++r) v[b * SA + r] = cmul_w(v[b * SA + r], tw[r * 32 + tj + SA * b]);
+        for (int r = 1; r < SA; ++r) v[b * SA + r] = cmul_w(v[b * SA + r], tw[(r - 1) * 32 + tj + SA * b]);
         dftp<SA, 1, false, false>(v + b * SA, y + b * SA);
         C2 p[CH];
         p[0] = base;
@@ -487,7 +491,7 @@ __global__ void __launch_bounds__(32 * WARPS, WARPS == 4 ? 3 : 1) k_series(const
 #pragma unroll
       for (int b = 0; b < 32 / SB; ++b) {
 #pragma unroll
-        for (int r = 1; r < SB; ++r) v[b * SB + r] = cmul_w(v[b * SB + r], tw[r * (N2 / N1) * 32 + tj + SB * b]);
+        for (int r = 1; r < SB; ++r) v[b * SB + r] = cmul_w(v[b * SB + r], tw[(r * (N2 / N1) - 1) * 32 + tj + SB * b]);
         dftp<SB, 1, false, true>(v + b * SB, y + b * SB);
 #pragma unroll
         for (int kk = 0; kk < SB / 2; ++kk) z[b * (SB / 2) + kk] = y[b * SB + SB / 2 + kk];
@@ -635,7 +639,7 @@ int launch(Args a, int rows_ws, cudaStream_t st) {
   auto kern = k_series<LOG2N, WARPS, KIND>;
   RB_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmem));
   const int64_t items = (int64_t)S::ITEMS * a.nvec;
-  const int grid = (int)std::min<int64_t>(2 * items, sm_count() * (WARPS == 4 ? 3 : 1));
+  const int grid = (int)std::min<int64_t>(2 * items, sm_count() * S::kCtas);
   // A row is complete one row's items and the items in flight (half of every CTA's current and next) after its
   // first item; the ring holds the rows between the first A item and the last B item in flight.
   const auto rows_of = [&](int64_t t) { return (int)((t + S::ITEMS - 1) / S::ITEMS); };
