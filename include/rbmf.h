@@ -424,9 +424,10 @@ int rb_tune_stage1(const rb_filter_desc* desc, const rb_basis* basis, const floa
  * rb_filter / rb_filter_batch / rb_filter_plain). Few rows take two four-step passes, which have
  * RB_FFT_VARIANTS schedules (columns per CTA of the two passes, and the megabytes of the intermediate
  * that are to stay in L2): every one is timed on this desc's basis and s_hat, and the fastest is
- * remembered for the passes of (n, w) in a process-wide table (variant 0 when untuned). Many rows (2^22
- * points in all from n = 2^17 on, 2^23 from n = 2^14 on) take one fused launch, which has one schedule:
- * its time fills times_ms, *chosen is 0 and nothing is remembered. Measurement support, not in the paper.
+ * remembered for the passes of (n, w) in a process-wide table (variant 0 when untuned). Many rows (from
+ * 2^22 points in all at n = 2^17 and more, from 2^23 points at n = 2^14 and more) take one fused launch, which
+ * has one schedule: its time fills times_ms, *chosen is 0 and nothing is remembered. Measurement support, not
+ * in the paper.
  *   s_hat: [n/2] complex device (rb_whiten output). times_ms: HOST [RB_FFT_VARIANTS] mean ms of one
  *   basis filter. chosen: HOST, the selected variant. Synchronises `stream`.
  *   Errors: RB_ERR_BAD_INPUT (NULL argument, basis not matching desc), RB_ERR_OOM (workspace),

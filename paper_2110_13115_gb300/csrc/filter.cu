@@ -642,12 +642,26 @@ static int launch_b(const rb::Geometry& g, const PassBArgs& a, const rb::Tables&
 }
 
 // Whether nvec rows of n points go through the fused launch (series.cuh) or the two radix-16 passes. The fused launch
-// has the higher rate (2.8 against 4.8 us a row at n = 2^19) and a longer way to its first result (two whole items in
-// turn, about 20 us against 8 us), so the line is the work at which they meet, measured with rb_basis_filter, w = 8
-// (fused / radix-16, us): 2^19 x 4 rows 34 / 29, x 8 45 / 45, x 16 67 / 82; 2^17 x 32 39 / 38, x 64 59 / 72;
-// 2^16 x 64 38 / 33, x 128 60 / 64; 2^14 x 128 31 / 23.
-bool use_fused(const rb::Geometry& g, int64_t nvec) {
-  return g.n >= (1 << 14) && g.n * nvec >= (int64_t)(g.n >= (1 << 17) ? 1 << 22 : 1 << 23) && rb::fft_fused_enabled();
+// has the higher rate (2.6 against 4.8 us a row at n = 2^19) and a longer way to its first result (two whole items in
+// turn, about 20 us against 8 us), so the line is the work at which they meet. rb_basis_filter, w = 8, L2 flushed before
+// each call (fused / radix-16, us): 2^19 x 8 rows 47 / 50, x 16 68 / 88; 2^17 x 32 43 / 43, x 64 61 / 74; 2^16 x 128 62 / 65,
+// x 256 100 / 122; 2^14 x 512 66 / 64, x 1024 99 / 117. Bins of one sample give the second pass less to do: at n = 2^14 and
+// w = 1, 66 / 59 at 512 rows, 101 / 109 at 1024.
+bool use_fused(const rb::Geometry& g, int64_t nvec, int w) {
+  const int64_t line = g.n >= (1 << 17) ? 1 << 22 : g.n == (1 << 14) && w == 1 ? 3 << 22 : 1 << 23;
+  return g.n >= (1 << 14) && g.n * nvec >= line && rb::fft_fused_enabled();
+}
+
+// The same for the first stage by templates, whose rows come from the pass that folds them. Folding in the first radix-16
+// pass costs more than that pass, so the fused launch wins sooner (w = 2 and 8, M = n / w points, fused / radix-16, us):
+// 2^14 x 128 97 / 94 and 108 / 112, x 256 107 / 109 and 129 / 139; 2^15 x 64 94 / 98 and 111 / 124; 2^16 x 32 96 / 101 and
+// 129 / 141; 2^17 x 16 101 / 112 and 157 / 207; 2^18 x 8, w = 2 117 / 127; 2^19 x 4 143 / 148. Without a fold (lowpass) the
+// radix-16 pass forms the product on its way and the pass before the fused launch is so much more traffic: 2^14 x 4096
+// 668 / 456, 2^15 x 2048 628 / 498, 2^16 x 1024 635 / 516, 2^17 x 256 349 / 319, 2^18 x 128 359 / 341; only 2^19 x 16
+// 146 / 163, x 64 385 / 438, where 8 rows are 113 / 112.
+bool use_fused_fold(const rb::Geometry& gm, int64_t T, bool lowpass) {
+  const int64_t line = lowpass ? 1 << 23 : gm.n == (1 << 14) ? 1 << 22 : 1 << 21;
+  return gm.n >= (lowpass ? 1 << 19 : 1 << 14) && gm.n * T >= line && rb::fft_fused_enabled();
 }
 
 std::atomic<int> g_withhold{0};  // fused launches left whose part B waits in vain (failure-detection test)
@@ -729,7 +743,7 @@ int whiten(const Geometry& g, const Workspace& ws, const float* strain, float2* 
 
 static int bank_filter_v(const Geometry& g, const Workspace& ws, const float2* rows, int64_t nvec,
                          const float2* shat, float2* beta, float2* bavg, int w, const FftVariant& v, cudaStream_t st) {
-  if (use_fused(g, nvec)) {
+  if (use_fused(g, nvec, w)) {
     rbseries::Args a{};
     a.rows = rows;
     a.shat = shat;
@@ -783,7 +797,7 @@ int tune_fft(const Geometry& g, const Workspace& ws, const float2* rows, int64_t
   RB_CUDA_TRY(cudaEventCreate(&e1));
   // rows that take the fused launch have nothing to choose: one time serves for all, and the choice of the radix-16
   // passes, which fewer rows of this n and w take, stays what it was
-  const bool one = use_fused(g, nvec);
+  const bool one = use_fused(g, nvec, w);
   int rc = RB_OK, best = 0;
   for (int v = 0; v < (one ? 1 : RB_FFT_VARIANTS) && rc == RB_OK; ++v) {
     const int reps = 3;
@@ -818,7 +832,7 @@ int plain_filter(const Geometry& g, const Workspace& ws, const float2* tmpl, int
                  int w, float thr2, int64_t sample_offset, int block_id, rb_trigger* trig, int64_t cap,
                  cudaStream_t st) {
   const FftVariant& v = kFftVariants[fft_variant_for(g.n, w)];
-  if (use_fused(g, T)) {
+  if (use_fused(g, T, w)) {
     rbseries::Args a{};
     a.rows = tmpl;
     a.shat = shat;
@@ -856,7 +870,7 @@ int plain_filter(const Geometry& g, const Workspace& ws, const float2* tmpl, int
 int init_gfold(const Geometry& gm, int64_t T, const float2* shat, float2* gfold, int64_t n, int w, cudaStream_t st) {
   // four values a thread; the fused transforms take the weights times s_hat
   const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((n / 2 + 511) / 512, 1216));
-  k_gfold<<<(int)blocks, 128, 0, st>>>(use_fused(gm, T) ? shat : nullptr, gfold, n, w);
+  k_gfold<<<(int)blocks, 128, 0, st>>>(use_fused_fold(gm, T, false) ? shat : nullptr, gfold, n, w);
   RB_LAUNCH_CHECK();
   return RB_OK;
 }
@@ -865,7 +879,7 @@ int folded_stage1(const Geometry& gm, const Workspace& wm, const float2* tmpl, i
                   float thr2, int block_id, rb_candidate* cand, int64_t cap, const float2* gfold, float2* folded, int rows,
                   cudaStream_t st, bool lowpass) {
   const FftVariant& v = kFftVariants[fft_variant_for(gm.n, 1)];
-  if (use_fused(gm, T)) {
+  if (use_fused_fold(gm, T, lowpass)) {
     const int64_t M = gm.n, half = M * w / 2;
     const float2* u = lowpass ? shat : gfold;
     const int aligned = ((uintptr_t)tmpl & 15) == 0;
