@@ -149,6 +149,7 @@ HOST_HOOKS = {
     "rbx_set_stage2_ring": (C.c_int, [C.c_int]),
     "rbx_set_stage2_tc_piece": (C.c_int, [C.c_int]),
     "rbx_set_stage2_tc_windows": (C.c_int, [C.c_int]),
+    "rbx_refine_division": (C.c_int, [C.c_int64, _P, _P, _P, _P]),
     "rbx_mma_sync_rate": (C.c_int, [C.c_int, C.POINTER(C.c_double)]),
 }
 

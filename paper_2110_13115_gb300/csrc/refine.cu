@@ -97,6 +97,18 @@ struct RefArgs {
   double alpha0, alpha_max;
 };
 
+// --- division -----------------------------------------------------------------------------------
+// Quotients and reciprocals by the corrections with fused multiply-adds of Markstein (IBM J. Res. Dev. 34, 1990): the
+// residual of a guess within a few units in the last place is exact, and its correction rounds once, so the result is the
+// rounded quotient unless that lies within some 2^-50 units of a tie.
+// x / d by the rounded r = 1 / d
+__host__ __device__ __forceinline__ double quotient(double x, double d, double r) {
+  const double q = x * r;
+  return fma(fma(-d, q, x), r, q);
+}
+// 1 / v
+__host__ __device__ __forceinline__ double reciprocal(double v, double guess) { return fma(guess, fma(-v, guess, 1.0), guess); }
+
 // --- pairs ------------------------------------------------------------------------------------
 struct Pair {
   float h, l;
@@ -341,7 +353,7 @@ __device__ void evaluate(const RefArgs& a, const cg::cluster_group& cluster, con
       }
       const double2 vt = __ldg(a.v + j);
       const double vv = m13 * vt.x, guess = r13 * vt.y;  // 1 / vv within two units in the last place
-      const double iv = fma(guess, fma(-vv, guess, 1.0), guess);
+      const double iv = reciprocal(vv, guess);
       const double iv2 = iv * iv, iv3 = iv2 * iv, iv5 = iv3 * iv2;
       double phase = __ldg(a.x + j) * tc - phic - 0.25 * kPi;
       if constexpr (GRAD) {  // (rounded as in the ascent)
@@ -511,11 +523,6 @@ __global__ void __launch_bounds__(kThreads, MODE == R_EVAL ? 8 : 5) k_refine(Ref
 }
 
 // --- the ascent ------------------------------------------------------------------------------------
-// x / d by the correctly rounded r = 1 / d: the residual of the first guess is exact and its correction rounds once.
-__device__ __forceinline__ double quotient(double x, double d, double r) {
-  const double q = __dmul_rn(x, r);
-  return __fma_rn(__fma_rn(-d, q, x), r, q);
-}
 // a sine or cosine (zero, normal or NaN) in FP64 by its bits: conversions run at the FP64 rate
 __device__ __forceinline__ double widen(float x) {
   const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
@@ -568,7 +575,7 @@ __device__ void evaluate_fp64(const RefArgs& a, const cg::cluster_group& cluster
     const double2 vt = __ldg(a.v + j), sh = __ldg(a.sh + j);
     const double x = __ldg(a.x + j), am = __ldg(a.amp + j);
     const double vv = __dmul_rn(m13, vt.x), guess = r13 * vt.y;  // 1 / vv within two units in the last place
-    const double iv = __fma_rn(guess, __fma_rn(-vv, guess, 1.0), guess);
+    const double iv = reciprocal(vv, guess);
     const double iv2 = __dmul_rn(iv, iv), iv3 = __dmul_rn(iv2, iv), iv5 = __dmul_rn(iv3, iv2);
     double in = __fma_rn(c2, iv3, iv5);
     if (PN3) in = __fma_rn(c3, iv2, in);
@@ -907,3 +914,12 @@ int rb_refine(const rb_refine_desc* d, const float* s_hat, const double* psd, do
 }
 
 }  // extern "C"
+
+// Host-only test hook (not part of the C ABI): the quotients a / b and the reciprocals 1 / (a b) as the kernels form them.
+extern "C" int rbx_refine_division(int64_t n, const double* a, const double* b, double* q, double* inv) {
+  for (int64_t i = 0; i < n; ++i) {
+    q[i] = quotient(a[i], b[i], 1.0 / b[i]);
+    inv[i] = reciprocal(a[i] * b[i], (1.0 / a[i]) * (1.0 / b[i]));
+  }
+  return 0;
+}
