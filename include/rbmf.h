@@ -585,9 +585,12 @@ typedef struct rb_refine_desc {
  *   J(theta) = |Z|^2 / sigma^2,                  sigma^2 = sum_j |g_j|^2,
  * over the support f_low <= f_j < f_isco(theta_start), 0 < j < n/2, frozen at the starting point (so
  * sigma does not depend on theta). Psi is evaluated in FP64 and reduced modulo 2 pi before FP32
- * sin/cos; the terms and their sums are kept in pairs of FP32 values (48 bits and more), relative to the
- * largest term of the candidate's own support, so that PSD values and data of any size may lie in the
- * block. One CTA per candidate; the template is recomputed in every pass, no per-template series is stored.
+ * sin/cos; the terms and their sums are kept to more than FP64's precision in rb_refine_eval and
+ * rb_refine_adjoint (unevaluated sums of three FP32 values, relative to the largest term of the candidate's
+ * own support, so that PSD values and data of any size may lie in the block) and in FP64 in rb_refine. A
+ * candidate is shared by up to eight CTAs (two in rb_refine), and its results have the same bits whatever
+ * other candidates are in the call. The template is recomputed in every pass, no per-template series is
+ * stored; the workspace holds tables over the frequencies, 44 to 52 bytes per sample.
  *   s_hat: [n/2] complex device (rb_whiten output).  psd: [n/2+1] float64 device.
  *   theta: [n_cand][4] float64 device.  workspace: at least rb_refine_workspace_bytes(desc) bytes.
  */

@@ -9,21 +9,25 @@
 // them (four divisions among them). FP64 is left to the phase, which needs it (Psi reaches 1e5 rad and more and is
 // rounded to FP32 only after its reduction modulo 2 pi), in 16 operations: 1 / v comes from a table of 1 / vf and one
 // Newton step that rounds it correctly, 2 pi f from a table, the reduction multiplies by 1 / (2 pi). The rest runs in FP32
-// pairs (an unevaluated sum hi + lo, 48 bits; the products and sums are the classical error-free ones): the term
-// amp s_hat e^(i Psi), and its sums. The derivatives of Psi are linear in f, F5 = (pi f)^(-5/3), F3 = (pi f)^(-1) and
+// with values in three parts (an unevaluated sum, 72 bits; the products and sums are the classical error-free ones): the
+// term amp s_hat e^(i Psi), and its sums. The derivatives of Psi are linear in f, F5 = (pi f)^(-5/3), F3 = (pi f)^(-1) and
 // F2 = (pi f)^(-2/3) with coefficients that are constant over the points, so a pass sums the terms and their moments
 // with those four, and one thread forms the gradient.
+// Precision. Against sums in 64-bit mantissas over the same sines and cosines, relative to the norm of what is summed
+// (rms over candidates; mc, eta, t_c, phi_c): n = 2^14 3.5, 2.3, 1.6, 1.1 x 1e-16, where plain FP64 had 5.2, 23.9, 2.6,
+// 2.9; n = 2^16, third order 7.2, 3.0, 2.7, 1.7 (8.6, 5.9, 5.2, 5.1); n = 2^19 7.6, 5.0, 2.9, 2.8 (10.3, 24.6, 6.6, 6.8). With
+// pairs of values (48 bits) it was 20 to 40 throughout.
 // Range. amp goes with the PSD and the units of the strain over hundreds of decades, s_hat over FP32's: the products
-// amp s_hat are formed in FP64 and kept as pairs of order one with an exponent of their own (four bytes a frequency),
-// and a candidate takes them relative to the largest exponent of its own support. So neither a bin outside the support
-// nor another candidate moves them, and what is lost is 2^-126 of the support's largest value and below.
-// Measured (FP64 issue bounds it, 16 operations a point): value and gradient of 500 candidates at n = 2^19 1.48 ms
-// against 4.39 ms with every point in FP64. A phase in pairs too would take 0.65 ms and is as accurate, but it rounds to
-// another FP32 phase at one point in some thousands.
+// amp s_hat are formed in FP64 and kept as values of order one with an exponent of their own, and a candidate takes them
+// relative to the largest exponent of its own support. So neither a bin outside the support nor another candidate moves
+// them, and what is lost is 2^-126 of the support's largest value and below.
+// Measured (FP64 issue bounds it, 16 operations a point; the FP32 work beside it is twice that of pairs and nearly free):
+// value and gradient of 500 candidates at n = 2^19 1.55 ms against 4.39 ms with every point in FP64 and 1.51 ms with
+// pairs. A phase in pairs too would take 0.65 ms, but it rounds to another FP32 phase at one point in some thousands.
 //
 // The ascent stays in FP64 (k_refine_ascend): a last digit of the gradient is a last digit of theta, which moves the FP32
-// phase of a few points, and so J by 1e-9, and now and then the choice of a step; with pairs, J came out up to 6e-9 (norm
-// over the candidates) from what this library gave before. It does the same roundings in the same order (the FMAs
+// phase of a few points, and so J by 1e-9, and now and then the choice of a step; with sums in FP32 parts, J came out up to
+// 6e-9 (norm over the candidates) from what this library gave before. It does the same roundings in the same order (the FMAs
 // are written out, so that no compiler regroups them) in 45 FP64 operations a point instead of about 90: quotients by
 // reciprocals formed once per pass, 1 / v as above, tables, sine and cosine widened by their bits, no sums twice.
 // 512 candidates x 20 steps at n = 2^17: 7.11 ms against 15.3 ms, bit for bit.
@@ -67,12 +71,13 @@ struct RefArgs {
   const float2* shat;
   const double* psd;
   Header* head;
-  float4* w;      // 2^-e amp s_hat as pairs: (re hi, im hi, re lo, im lo), amp = f^(-7/6) sqrt(4 df / S)
-  int* e;         // the exponent of its larger part
+  float4* w;      // 2^-e amp s_hat in three parts: (re h, im h, re m, im m), amp = f^(-7/6) sqrt(4 df / S)
+  float4* wl;     // (re l, im l, e as an integer: the exponent of the larger part)
   double2* v;     // (vf, 1 / vf), vf = (pi f)^(1/3)
   double* x;      // 2 pi f
-  float4* g;      // (F5 hi, F5 lo, F3 hi, F3 lo) over their values at the band's first frequency
-  float2* g2;     // (F2 hi, F2 lo), the same
+  float4* g;      // (F5 h, F5 m, F3 h, F3 m) over their values at the band's first frequency
+  float2* gl;     // (F5 l, F3 l)
+  float4* g2;     // (F2 h, F2 m, F2 l)
   double* amp2;   // amp^2, zero below the band
   double* chunk;  // sums of amp2 over blocks of kThreads frequencies
   int* top;       // the largest e of these blocks
@@ -109,13 +114,17 @@ __host__ __device__ __forceinline__ double quotient(double x, double d, double r
 // 1 / v
 __host__ __device__ __forceinline__ double reciprocal(double v, double guess) { return fma(guess, fma(-v, guess, 1.0), guess); }
 
-// --- pairs ------------------------------------------------------------------------------------
-struct Pair {
-  float h, l;
+// --- values in three parts ------------------------------------------------------------------------
+// An unevaluated sum of three FP32 values, 72 bits: it holds an FP64 value exactly.
+struct Three {
+  float h, m, l;
 };
-__device__ __forceinline__ Pair to_pair(double x) {
+__device__ __forceinline__ Three to_three(double x) {
   const float h = (float)x;
-  return {h, isfinite(h) ? (float)(x - (double)h) : 0.f};
+  if (!isfinite(h)) return {h, 0.f, 0.f};
+  const double r = x - (double)h;
+  const float m = (float)r;
+  return {h, m, (float)(r - (double)m)};
 }
 // s + e = a + b exactly (Knuth)
 __device__ __forceinline__ float two_sum(float a, float b, float& e) {
@@ -123,28 +132,41 @@ __device__ __forceinline__ float two_sum(float a, float b, float& e) {
   e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
   return s;
 }
-// Sums are kept in three parts: a pair's low part collects the rounding errors of every addition, and its own
-// rounding would cost a digit and a half over a pass (1.6e-14 of the terms' norm against 2e-15).
-struct Sum {
-  float h, m, l;
-};
-__device__ __forceinline__ void add(Sum& s, float h, float l) {
-  float e1, e2, e3;
-  s.h = two_sum(s.h, h, e1);
-  const float x = two_sum(e1, l, e2);
-  s.m = two_sum(s.m, x, e3);
-  s.l = __fadd_rn(s.l, __fadd_rn(e2, e3));
+// p + e = a b exactly
+__device__ __forceinline__ float two_prod(float a, float b, float& e) {
+  const float p = __fmul_rn(a, b);
+  e = __fmaf_rn(a, b, -p);
+  return p;
 }
-__device__ __forceinline__ Sum shuffle_xor(const Sum& s, int off) {
+__device__ __forceinline__ void add(Three& s, const Three& o) {
+  float e1, e2, e3;
+  s.h = two_sum(s.h, o.h, e1);
+  const float x = two_sum(e1, o.m, e2);
+  s.m = two_sum(s.m, x, e3);
+  s.l = __fadd_rn(s.l, __fadd_rn(__fadd_rn(e2, e3), o.l));
+}
+__device__ __forceinline__ Three shuffle_xor(const Three& s, int off) {
   return {__shfl_xor_sync(0xffffffffu, s.h, off), __shfl_xor_sync(0xffffffffu, s.m, off), __shfl_xor_sync(0xffffffffu, s.l, off)};
 }
-__device__ __forceinline__ void add(Sum& s, const Sum& o) {
-  add(s, o.h, o.m);
-  s.l = __fadd_rn(s.l, o.l);
+__device__ __forceinline__ Three mul(const Three& a, float b) {
+  float e1, e2, e3;
+  const float p = two_prod(a.h, b, e1), q = two_prod(a.m, b, e2), m = two_sum(e1, q, e3);
+  return {p, m, __fmaf_rn(a.l, b, __fadd_rn(e2, e3))};
 }
-__device__ __forceinline__ Pair mul(Pair a, float bh, float bl) {
-  const float p = __fmul_rn(a.h, bh);
-  return {p, __fmaf_rn(a.l, bh, __fmaf_rn(a.h, bl, __fmaf_rn(a.h, bh, -p)))};
+__device__ __forceinline__ Three mul(const Three& a, const Three& b) {
+  float e1, e2, e3, e4, e5;
+  const float p = two_prod(a.h, b.h, e1), q = two_prod(a.h, b.m, e2), r = two_prod(a.m, b.h, e3);
+  const float s = two_sum(q, r, e4), m = two_sum(s, e1, e5);
+  return {p, m, __fmaf_rn(a.h, b.l, __fmaf_rn(a.m, b.m, __fmaf_rn(a.l, b.h, __fadd_rn(__fadd_rn(e2, e3), __fadd_rn(e4, e5)))))};
+}
+// a b + c d
+__device__ __forceinline__ Three dot(const Three& a, float b, const Three& c, float d) {
+  float e1, e2, e3, e4, e5, e6, e7, e8, e9;
+  const float p = two_prod(a.h, b, e1), q = two_prod(c.h, d, e2), h = two_sum(p, q, e3);
+  const float r = two_prod(a.m, b, e4), t = two_prod(c.m, d, e5);
+  const float x = two_sum(e1, e2, e6), y = two_sum(r, t, e7), z = two_sum(x, y, e8), m = two_sum(z, e3, e9);
+  const float l = __fadd_rn(__fadd_rn(e4, e5), __fadd_rn(__fadd_rn(e6, e7), __fadd_rn(e8, e9)));
+  return {h, m, __fmaf_rn(a.l, b, __fmaf_rn(c.l, d, l))};
 }
 
 // The exponent e of a complex value: its larger part lies in [2^e, 2^(e + 1)) (zero and below FP64's normal range:
@@ -206,8 +228,10 @@ __device__ __forceinline__ int block_max(int v, int* red) {
 
 constexpr int kNoExponent = -(1 << 20);  // of frequencies outside the band
 
-// The tables on [jlo, jmax): everything is a power of y = j^(-1/6) (an FP32 estimate and two Newton steps in
-// FP64: the error 3.5 e^2 of a step takes 1e-6 below the rounding of FP64).
+// The tables on [jlo, jmax): everything is a power of y = j^(-1/6) (an FP32 estimate and a Newton step in FP64, which
+// takes its error from 1e-6 to 1e-11). The powers' roundings are kept (x2 .. x10) and so is what y itself is off by, d
+// relative to it: with both the table values are rounded once or twice, where a seventh or a tenth power of a rounded y would
+// be off by several units, as much as the sums.
 __global__ void __launch_bounds__(kThreads) k_refine_tables(RefArgs a) {
   __shared__ double red[kThreads / 32];
   __shared__ int red_e[kThreads / 32];
@@ -216,32 +240,41 @@ __global__ void __launch_bounds__(kThreads) k_refine_tables(RefArgs a) {
     const int64_t j = c * kThreads + threadIdx.x;
     double a2 = 0.0;
     int e = kNoExponent;
+    float4 lows = make_float4(0.f, 0.f, __int_as_float(kNoExponent), 0.f);
     if (j >= a.jlo && j < jmax) {
-      const double f = j * a.df, x = (double)(int)j;
+      const double f = j * a.df, x = (double)(int)j, S = a.psd[j];
       double y = (double)exp2f(log2f((float)(int)j) * (-1.f / 6.f));
-#pragma unroll
-      for (int it = 0; it < 2; ++it) {
+      {
         const double y2 = y * y, y6 = y2 * y2 * y2;
         y = y * (fma(-x, y6, 7.0) * (1.0 / 6.0));
       }
-      const double y2 = y * y, y4 = y2 * y2, y6 = y4 * y2, y10 = y6 * y4;
-      const double am = a.amp0 * (y6 * y) * rsqrt(a.psd[j]);
+      const double y2 = y * y, x2 = fma(y, y, -y2), y3 = y2 * y, x3 = fma(x2, y, fma(y2, y, -y3));
+      const double y4 = y2 * y2, x4 = fma(2.0 * y2, x2, fma(y2, y2, -y4)), y6 = y3 * y3, x6 = fma(2.0 * y3, x3, fma(y3, y3, -y6));
+      const double d = (fma(-x, y6, 1.0) - x * x6) * (1.0 / 6.0);
+      const double y7 = y6 * y, x7 = fma(x6, y, fma(y6, y, -y7));
+      const double y10 = y6 * y4, x10 = fma(x6, y4, fma(y6, x4, fma(y6, y4, -y10)));
+      // 1 / sqrt(S) = s (1 + h)
+      const double s = rsqrt(S), u = S * s, h = 0.5 * (fma(-u, s, 1.0) - fma(S, s, -u) * s);
+      const double am = (a.amp0 * s) * (y7 + fma(fma(7.0, d, h), y7, x7));
       const float2 sh = a.shat[j];
       const double wr = am * (double)sh.x, wi = am * (double)sh.y;
       e = exponent(wr, wi);
-      const Pair re = to_pair(scalbn(wr, -e)), im = to_pair(scalbn(wi, -e));
-      const Pair f5 = to_pair(a.r53 * y10), f3 = to_pair(a.r33 * y6), f2 = to_pair(a.r23 * y4);
+      const Three re = to_three(scalbn(wr, -e)), im = to_three(scalbn(wi, -e));
+      const Three f5 = to_three(a.r53 * (y10 + fma(10.0 * d, y10, x10))), f3 = to_three(a.r33 * (y6 + fma(6.0 * d, y6, x6))),
+                  f2 = to_three(a.r23 * (y4 + fma(4.0 * d, y4, x4)));
       const double vf = cbrt(kPi * f);
       a.v[j] = make_double2(vf, 1.0 / vf);
       a.x[j] = 2.0 * kPi * f;
-      a.w[j] = make_float4(re.h, im.h, re.l, im.l);
-      a.g[j] = make_float4(f5.h, f5.l, f3.h, f3.l);
-      a.g2[j] = make_float2(f2.h, f2.l);
+      a.w[j] = make_float4(re.h, im.h, re.m, im.m);
+      a.g[j] = make_float4(f5.h, f5.m, f3.h, f3.m);
+      a.gl[j] = make_float2(f5.l, f3.l);
+      if (a.pn >= 3) a.g2[j] = make_float4(f2.h, f2.m, f2.l, 0.f);
+      lows = make_float4(re.l, im.l, __int_as_float(e), 0.f);
       a2 = am * am;
     }
     if (j < a.half) {
       a.amp2[j] = a2;
-      a.e[j] = e;
+      a.wl[j] = lows;
     }
     a2 = block_sum(a2, red);
     e = block_max(e, red_e);
@@ -303,7 +336,7 @@ struct Sums {
 
 // Sums of V values over a warp into out[V]: halves of the list are exchanged while there is more than one value left.
 template <int V>
-__device__ __forceinline__ void warp_sums(Sum (&v)[V], double* out) {
+__device__ __forceinline__ void warp_sums(Three (&v)[V], double* out) {
   const int lane = threadIdx.x & 31;
   int first = 0;
 #pragma unroll
@@ -314,7 +347,7 @@ __device__ __forceinline__ void warp_sums(Sum (&v)[V], double* out) {
       first += up ? keep : 0;
 #pragma unroll
       for (int i = 0; i < keep; ++i) {
-        const Sum give = up ? v[i] : v[i + keep];
+        const Three give = up ? v[i] : v[i + keep];
         v[i] = up ? v[i + keep] : v[i];
         add(v[i], shuffle_xor(give, off));
       }
@@ -343,13 +376,15 @@ __device__ void evaluate(const RefArgs& a, const cg::cluster_group& cluster, con
   __syncthreads();  // (red may still be read)
 #pragma unroll 1
   for (int q = 0; q < own; ++q) {
-    Sum v[V] = {}, v2[2] = {};
+    Three v[V] = {}, v2[2] = {};
 #pragma unroll 2
     for (int j = (int)a.jlo + (rank * own + q) * kThreads + (int)threadIdx.x; j < (int)jhi; j += a.strands * kThreads) {  // (< 2^20)
-      float4 w = __ldg(a.w + j);
+      Three wr, wi;
       {  // to the support's scale: 2^(e - top), nothing below 2^-126
-        const float unit = __int_as_float((max(__ldg(a.e + j) - top, -127) + 127) << 23);
-        w = make_float4(w.x * unit, w.y * unit, w.z * unit, w.w * unit);
+        const float4 w = __ldg(a.w + j), l = __ldg(a.wl + j);
+        const float unit = __int_as_float((max(__float_as_int(l.z) - top, -127) + 127) << 23);
+        wr = {w.x * unit, w.z * unit, l.x * unit};
+        wi = {w.y * unit, w.w * unit, l.y * unit};
       }
       const double2 vt = __ldg(a.v + j);
       const double vv = m13 * vt.x, guess = r13 * vt.y;  // 1 / vv within two units in the last place
@@ -369,36 +404,26 @@ __device__ void evaluate(const RefArgs& a, const cg::cluster_group& cluster, con
       float sn, cs;
       sincosf(psi, &sn, &cs);
       // term = w exp(i Psi)
-      Pair t[2];
-      float e;
-      {
-        const float p = __fmul_rn(w.x, cs), q = __fmul_rn(w.y, sn);
-        t[0].h = two_sum(p, -q, e);
-        t[0].l = __fadd_rn(e, __fsub_rn(__fmaf_rn(w.z, cs, __fmaf_rn(w.x, cs, -p)), __fmaf_rn(w.w, sn, __fmaf_rn(w.y, sn, -q))));
+      const Three t[2] = {dot(wr, cs, wi, -sn), dot(wr, sn, wi, cs)};
+      Three f5, f3, f2;
+      if constexpr (GRAD) {
+        const float4 g = __ldg(a.g + j);
+        const float2 l = __ldg(a.gl + j);
+        f5 = {g.x, g.y, l.x};
+        f3 = {g.z, g.w, l.y};
       }
-      {
-        const float p = __fmul_rn(w.x, sn), q = __fmul_rn(w.y, cs);
-        t[1].h = two_sum(p, q, e);
-        t[1].l = __fadd_rn(e, __fadd_rn(__fmaf_rn(w.z, sn, __fmaf_rn(w.x, sn, -p)), __fmaf_rn(w.w, cs, __fmaf_rn(w.y, cs, -q))));
+      if constexpr (GRAD && PN3) {
+        const float4 g = __ldg(a.g2 + j);
+        f2 = {g.x, g.y, g.z};
       }
-      float4 g;
-      float2 g2;
-      if constexpr (GRAD) g = __ldg(a.g + j);
-      if constexpr (GRAD && PN3) g2 = __ldg(a.g2 + j);
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
-        add(v[c], t[c].h, t[c].l);
+        add(v[c], t[c]);
         if constexpr (GRAD) {
-          const float fj = (float)j;  // exact
-          const float p = __fmul_rn(t[c].h, fj);
-          add(v[2 + c], p, __fmaf_rn(t[c].l, fj, __fmaf_rn(t[c].h, fj, -p)));
-          const Pair x5 = mul(t[c], g.x, g.y), x3 = mul(t[c], g.z, g.w);
-          add(v[4 + c], x5.h, x5.l);
-          add(v[6 + c], x3.h, x3.l);
-          if constexpr (PN3) {
-            const Pair x2 = mul(t[c], g2.x, g2.y);
-            add(v2[c], x2.h, x2.l);
-          }
+          add(v[2 + c], mul(t[c], (float)j));  // (exact)
+          add(v[4 + c], mul(t[c], f5));
+          add(v[6 + c], mul(t[c], f3));
+          if constexpr (PN3) add(v2[c], mul(t[c], f2));
         }
       }
     }
@@ -464,7 +489,7 @@ __device__ __forceinline__ int64_t support_end(const RefArgs& a, double mc0, dou
 }
 
 template <int MODE, bool PN3>
-__global__ void __launch_bounds__(kThreads, MODE == R_EVAL ? 8 : 5) k_refine(RefArgs a) {
+__global__ void __launch_bounds__(kThreads, MODE == R_EVAL ? 6 : 5) k_refine(RefArgs a) {
   // (of the cluster's first CTA: point, parts, s_jhi)
   __shared__ double red[kMaxRanks * (kThreads / 32) * 10], parts[kMaxRanks * 10];
   __shared__ int red_e[kThreads / 32];
@@ -493,7 +518,7 @@ __global__ void __launch_bounds__(kThreads, MODE == R_EVAL ? 8 : 5) k_refine(Ref
   const int64_t whole = jhi / kThreads, part = whole * kThreads + threadIdx.x;
   int top = kNoExponent;
   for (int64_t k = a.jlo / kThreads + threadIdx.x; k < whole; k += kThreads) top = max(top, a.top[k]);
-  if (part < jhi && part >= a.jlo) top = max(top, a.e[part]);
+  if (part < jhi && part >= a.jlo) top = max(top, __float_as_int(a.wl[part].z));
   top = block_max(top, red_e);
   double sig2 = 0.0;  // (the lead's thread 0)
   if (lead) {
@@ -718,8 +743,9 @@ __global__ void __launch_bounds__(kAscThreads / kAscRanks, 2 * kAscRanks) k_refi
 
 size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 
-// Workspace: header, then the tables over the frequencies. base == nullptr: only the size.
-size_t carve(int64_t half, char* base, RefArgs* a) {
+// Workspace: header, then the tables over the frequencies (88 bytes each, 104 with the phase's third order; the ascent
+// uses 48 of them). base == nullptr: only the size.
+size_t carve(int64_t half, int pn, char* base, RefArgs* a) {
   size_t off = 0;
   auto take = [&](size_t bytes) {
     char* p = base ? base + off : nullptr;
@@ -732,11 +758,12 @@ size_t carve(int64_t half, char* base, RefArgs* a) {
   a->v = (double2*)take(sizeof(double2) * half);
   a->x = (double*)take(sizeof(double) * half);
   a->g = (float4*)take(sizeof(float4) * half);
-  a->g2 = (float2*)take(sizeof(float2) * half);
+  a->gl = (float2*)take(sizeof(float2) * half);
+  a->g2 = (float4*)take(pn >= 3 ? sizeof(float4) * half : 0);
   a->amp2 = (double*)take(sizeof(double) * half);
   a->amp = a->amp2;
   a->chunk = (double*)take(sizeof(double) * ((half + kThreads - 1) / kThreads));
-  a->e = (int*)take(sizeof(int) * half);
+  a->wl = (float4*)take(sizeof(float4) * half);
   a->top = (int*)take(sizeof(int) * ((half + kThreads - 1) / kThreads));
   return off;
 }
@@ -759,7 +786,7 @@ int prepare(const rb_refine_desc* d, const float* shat, const double* psd, const
     return RB_ERR_OOM;
   }
   const int64_t half = d->n / 2;
-  carve(half, (char*)ws, &a);
+  carve(half, d->pn_order, (char*)ws, &a);
   a.shat = (const float2*)shat;
   a.psd = psd;
   a.theta_in = (const double*)theta;
@@ -863,7 +890,7 @@ extern "C" {
 size_t rb_refine_workspace_bytes(const rb_refine_desc* d) {
   if (!d || d->n < 2) return 0;
   RefArgs a{};
-  return carve(d->n / 2, nullptr, &a);
+  return carve(d->n / 2, d->pn_order, nullptr, &a);
 }
 
 int rb_refine_eval(const rb_refine_desc* d, const float* s_hat, const double* psd, const double* theta, double* J,
