@@ -866,18 +866,25 @@ int run(const RefArgs& a, cudaStream_t st) {
 }
 
 int ascend(const RefArgs& a, cudaStream_t st) {
-  if (a.n_cand > 0) {
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kAscRanks;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kAscRanks;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  constexpr int64_t kMost = ((int64_t)1 << 30) / kAscRanks;  // candidates of a launch (a grid has less than 2^31 CTAs)
+  for (int64_t c = 0; c < a.n_cand; c += kMost) {
+    RefArgs part = a;
+    part.n_cand = std::min(kMost, a.n_cand - c);
+    part.theta_in += 4 * c;
+    part.theta_out += 4 * c;
+    part.J += c;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(a.n_cand * kAscRanks));
+    cfg.gridDim = dim3((unsigned)(part.n_cand * kAscRanks));
     cfg.blockDim = dim3(kAscThreads / kAscRanks);
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    RB_CUDA_TRY(a.pn >= 3 ? cudaLaunchKernelEx(&cfg, k_refine_ascend<true>, a) : cudaLaunchKernelEx(&cfg, k_refine_ascend<false>, a));
+    RB_CUDA_TRY(part.pn >= 3 ? cudaLaunchKernelEx(&cfg, k_refine_ascend<true>, part)
+                             : cudaLaunchKernelEx(&cfg, k_refine_ascend<false>, part));
     RB_LAUNCH_CHECK();
   }
   return finish(a, st);
