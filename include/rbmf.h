@@ -280,9 +280,11 @@ int rb_filter_banks(const rb_filter_desc* descs, const rb_basis* bases, int32_t 
  *   templates: [T][n/2] complex whitened unit-norm templates (g_t / sigma_t, as rb_templates).
  *   strain: [n] float32.  psd: [n/2 + 1] float64.  desc: fs, n, w (2..16), n_templates, rho_i,
  *   cand_capacity, block_id used (k, precision, rho_ii ignored; mem must be 0).
- *   cand: [cand_capacity] output; n_cand (host). workspace: rb_folded_plan size. Synchronises `stream`.
+ *   cand: [cand_capacity] output; n_cand (host). workspace: rb_folded_plan size (up to 96 MB of the transforms'
+ *   intermediate and, for n / w >= 2^14, up to 64 MB of folded spectra). Synchronises `stream`.
  *   Errors: RB_ERR_BAD_INPUT (w < 2, NULL array, PSD), RB_ERR_UNSUPPORTED (n / w < 1024),
- *   RB_ERR_OOM (workspace), RB_ERR_OVERFLOW (more candidates than cand_capacity; *n_cand = count).
+ *   RB_ERR_OOM (workspace), RB_ERR_OVERFLOW (more candidates than cand_capacity; *n_cand = count),
+ *   RB_ERR_TIMEOUT (a bounded device-side wait ran out).
  */
 int rb_folded_plan(const rb_filter_desc* desc, size_t* workspace_bytes /* host */);
 int rb_stage1_folded(const rb_filter_desc* desc, const float* templates, const float* strain, const double* psd,
@@ -308,7 +310,8 @@ int rb_stage1_lowpass(const rb_filter_desc* desc, const float* templates, const 
  *   templates: [T][n/2] complex whitened unit-norm templates (g_t / sigma_t).
  *   strain, psd, trig, capacity, n_trig: as rb_filter (desc->k, w, rho_ii used; rho_i ignored).
  *   Errors: RB_ERR_BAD_INPUT (NULL array, negative capacity, PSD not finite and > 0 on 0 < j < n/2),
- *   RB_ERR_OOM (workspace), RB_ERR_OVERFLOW (more triggers than capacity; *n_trig = the count).
+ *   RB_ERR_OOM (workspace), RB_ERR_OVERFLOW (more triggers than capacity; *n_trig = the count),
+ *   RB_ERR_TIMEOUT (a bounded device-side wait ran out).
  */
 int rb_filter_plain(const rb_filter_desc* desc, const float* templates, const float* strain,
                     const double* psd, rb_trigger* trig, int64_t capacity, int64_t* n_trig,
