@@ -593,7 +593,7 @@ typedef struct rb_refine_desc {
  * own support, so that PSD values and data of any size may lie in the block) and in FP64 in rb_refine. A
  * candidate is shared by up to eight CTAs (two in rb_refine), and its results have the same bits whatever
  * other candidates are in the call. The template is recomputed in every pass, no per-template series is
- * stored; the workspace holds tables over the frequencies, 44 to 52 bytes per sample.
+ * stored; the workspace holds tables over the frequencies, 52 bytes per sample.
  *   s_hat: [n/2] complex device (rb_whiten output).  psd: [n/2+1] float64 device.
  *   theta: [n_cand][4] float64 device.  workspace: at least rb_refine_workspace_bytes(desc) bytes.
  */

@@ -743,9 +743,9 @@ __global__ void __launch_bounds__(kAscThreads / kAscRanks, 2 * kAscRanks) k_refi
 
 size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 
-// Workspace: header, then the tables over the frequencies (88 bytes each, 104 with the phase's third order; the ascent
-// uses 48 of them). base == nullptr: only the size.
-size_t carve(int64_t half, int pn, char* base, RefArgs* a) {
+// Workspace: header, then the tables over the frequencies (104 bytes each; the ascent uses 48 of them, value and adjoint 88
+// below the phase's third order: the size is a matter of n alone). base == nullptr: only the size.
+size_t carve(int64_t half, char* base, RefArgs* a) {
   size_t off = 0;
   auto take = [&](size_t bytes) {
     char* p = base ? base + off : nullptr;
@@ -759,7 +759,7 @@ size_t carve(int64_t half, int pn, char* base, RefArgs* a) {
   a->x = (double*)take(sizeof(double) * half);
   a->g = (float4*)take(sizeof(float4) * half);
   a->gl = (float2*)take(sizeof(float2) * half);
-  a->g2 = (float4*)take(pn >= 3 ? sizeof(float4) * half : 0);
+  a->g2 = (float4*)take(sizeof(float4) * half);
   a->amp2 = (double*)take(sizeof(double) * half);
   a->amp = a->amp2;
   a->chunk = (double*)take(sizeof(double) * ((half + kThreads - 1) / kThreads));
@@ -786,7 +786,7 @@ int prepare(const rb_refine_desc* d, const float* shat, const double* psd, const
     return RB_ERR_OOM;
   }
   const int64_t half = d->n / 2;
-  carve(half, d->pn_order, (char*)ws, &a);
+  carve(half, (char*)ws, &a);
   a.shat = (const float2*)shat;
   a.psd = psd;
   a.theta_in = (const double*)theta;
@@ -897,7 +897,7 @@ extern "C" {
 size_t rb_refine_workspace_bytes(const rb_refine_desc* d) {
   if (!d || d->n < 2) return 0;
   RefArgs a{};
-  return carve(d->n / 2, d->pn_order, nullptr, &a);
+  return carve(d->n / 2, nullptr, &a);
 }
 
 int rb_refine_eval(const rb_refine_desc* d, const float* s_hat, const double* psd, const double* theta, double* J,
